@@ -18,6 +18,7 @@
 #include "step_common.cuh"
 #include "step_grp.cuh"
 #include "step_small.cuh"
+#include "step_weak.cuh"
 
 namespace {
 
@@ -266,7 +267,7 @@ int step_device_mixed_grp(const double *src, double *dst, const double *masses, 
         cudaEventRecord(tm.second, g.stream);
         g.timers.push_back(tm);
     }
-    sakura::launch_apply_grp(dst, X, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
+    sakura::launch_apply_grp(dst, X, nullptr, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
                              g.d_status, g.stream);
     rc = launch_error();
     if (rc) return rc;
@@ -393,7 +394,7 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
         cudaEventRecord(tm.second, g.stream);
         g.timers.push_back(tm);
     }
-    sakura::launch_apply_grp(dst, X, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
+    sakura::launch_apply_grp(dst, X, nullptr, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
                              g.d_status, g.stream);
     rc = launch_error();
     if (rc) return rc;
@@ -408,6 +409,18 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
     return SAKURA_OK;
 }
 
+// Steps whose weakly perturbed pairs take the short solve of
+// kepler_weak.cuh: the FP64 form with the single-precision seed (where the
+// caller leaves the initial value to a float solve; with the other guesses
+// the iteration counts they are asked for stay theirs), the second-order map
+// it is written for, and a step whose products with ordinary velocities and
+// masses stay in float range.
+bool weak_form(int order, double tau)
+{
+    return g.cfg.precision == SAKURA_PREC_FP64 && g.cfg.guess == SAKURA_GUESS_FP32 &&
+           order == 2 && std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18;
+}
+
 // The FP64 form with each unordered pair once, in row-group phases
 // (step_grp.cu).  prepped: X (and X32) already hold this sub-step's drifted
 // state, written by the previous apply kernel; fuse: the apply kernel also
@@ -419,16 +432,17 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
     const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
     const bool seed = g.cfg.guess == SAKURA_GUESS_FP32;
-    int64_t blocks = g.cfg.grid_blocks > 0
-                         ? g.cfg.grid_blocks
-                         : (int64_t)g.sm_count *
-                               sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed);
+    const bool weak = !mixed && weak_form(order, dt);
+    int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks
+                     : (int64_t)g.sm_count *
+                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats)
+                                 : sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed));
     const sakura::GrpLayout L = sakura::make_grp_layout(n, sakura::kFp64GrpShape, blocks);
     // scratch: X[7][n] doubles, row partials [Hmax][6][n], column partials
     // [ng][6][n] and [blocks][6][32], then X32[10][n] floats (single-precision
-    // seed)
+    // seed) and the weak pairs' rows [4][n] of 16 bytes
     int rc = grow(g.partial, (size_t)(7 * n + (int64_t)(L.Hmax + L.ng) * 6 * n + blocks * 192 +
-                                      5 * n) *
+                                      5 * n + (weak ? 8 * n + 1 : 0)) *
                                  sizeof(double));
     if (rc) return rc;
     double *X = (double *)g.partial.ptr;
@@ -437,9 +451,15 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     parts.col = parts.row + (int64_t)L.Hmax * 6 * n;
     parts.colx = parts.col + (int64_t)L.ng * 6 * n;
     float *X32 = (seed || mixed) ? (float *)(parts.colx + blocks * 192) : nullptr;
+    // the weak rows, 16-byte aligned
+    const int64_t head = 12 * n + (int64_t)(L.Hmax + L.ng) * 6 * n + blocks * 192;
+    float4 *rows = weak ? (float4 *)(X + head + (head & 1)) : nullptr;
     const double drift = order == 2 ? 0.5 * dt : (order == 1 ? 0.0 : dt);
     const double post_drift = order == 2 ? 0.5 * dt : (order == 1 ? dt : 0.0);
-    if (!prepped) sakura::launch_prep_step(src, masses, X, X32, n, drift, g.d_status, g.stream);
+    if (!prepped && weak)
+        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, g.stream);
+    else if (!prepped)
+        sakura::launch_prep_step(src, masses, X, X32, n, drift, g.d_status, g.stream);
     sakura::StepArgs a;
     std::memset(&a, 0, sizeof(a));
     a.X = X;
@@ -468,13 +488,18 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
         tm = take_timer();
         cudaEventRecord(tm.first, g.stream);
     }
-    sakura::launch_pair_step_grp(a, L, parts, (int)blocks, stats, g.stream);
+    if (weak) {
+        const sakura::WeakStep ws{rows, 1.0 / dt};
+        sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, g.stream);
+    } else {
+        sakura::launch_pair_step_grp(a, L, parts, (int)blocks, stats, g.stream);
+    }
     g.group_launches += 1;
     if (timing) {
         cudaEventRecord(tm.second, g.stream);
         g.timers.push_back(tm);
     }
-    sakura::launch_apply_grp(dst, X, X32, parts, n, L, blocks, post_drift, fuse, next_drift,
+    sakura::launch_apply_grp(dst, X, X32, rows, parts, n, L, blocks, post_drift, fuse, next_drift,
                              g.d_status, g.stream);
     rc = launch_error();
     if (rc) return rc;
@@ -513,8 +538,10 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
     const bool seed = !df64 && g.cfg.guess == SAKURA_GUESS_FP32;
     const int64_t nb = (n + 31) / 32;
     const int64_t tiles = nb * (nb + 1) / 2;
-    const int bps = df64 ? sakura::pair_step_df64_blocks_per_sm(stats)
-                         : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
+    const bool weak = !df64 && !mixed && weak_form(order, dt);
+    const int bps = df64   ? sakura::pair_step_df64_blocks_per_sm(stats)
+                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats)
+                           : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
     // contiguous tile-step ranges for W <= T warps (step_common.cuh)
     const int64_t T = tiles * 32;
     int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks : (int64_t)g.sm_count * bps;
@@ -524,18 +551,24 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
     const int64_t nslots = nb * Smax;
     // scratch: X[7][n] doubles, tile partials [nslots][6][n] (doubles, or
     // double-words of two floats), then (df64) X3[20][n] or (seed) X32[10][n]
-    // floats
-    int rc = grow(g.partial, (size_t)(7 * n + nslots * 6 * n + (df64 ? 10 * n : 5 * n)) *
+    // floats and the weak pairs' rows [4][n] of 16 bytes
+    int rc = grow(g.partial, (size_t)(7 * n + nslots * 6 * n + (df64 ? 10 * n : 5 * n) +
+                                      (weak ? 8 * n + 1 : 0)) *
                                  sizeof(double));
     if (rc) return rc;
     double *X = (double *)g.partial.ptr;
     double *partial = X + 7 * n;
     float *X3 = (float *)(partial + nslots * 6 * n);
     float *X32 = (seed || mixed) ? X3 : nullptr;
+    // the weak rows, 16-byte aligned
+    const int64_t head = 12 * n + nslots * 6 * n;
+    float4 *rows = weak ? (float4 *)(X + head + (head & 1)) : nullptr;
     const double drift = order == 2 ? 0.5 * dt : (order == 1 ? 0.0 : dt);
     const double post_drift = order == 2 ? 0.5 * dt : (order == 1 ? dt : 0.0);
     if (df64)
         sakura::launch_prep_df64(src, masses, X, X3, n, drift, g.d_status, g.stream);
+    else if (!prepped && weak)
+        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, g.stream);
     else if (!prepped)
         sakura::launch_prep_step(src, masses, X, X32, n, drift, g.d_status, g.stream);
     sakura::StepArgs a;
@@ -576,6 +609,9 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         da.t = split_dw(dt);
         da.qtau = split_dw(a.post * dt);
         sakura::launch_pair_step_df64(a, da, Smax, T, (int)blocks, stats, g.stream);
+    } else if (weak) {
+        const sakura::WeakStep ws{rows, 1.0 / dt};
+        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, g.stream);
     } else {
         sakura::launch_pair_step_sym(a, Smax, T, (int)blocks, stats, g.stream);
     }
@@ -587,7 +623,7 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         sakura::launch_apply_df64(dst, X, partial, n, Smax, W, T, post_drift, g.d_status,
                                   g.stream);
     else
-        sakura::launch_apply_sym(dst, X, X32, partial, n, Smax, W, T, post_drift,
+        sakura::launch_apply_sym(dst, X, X32, rows, partial, n, Smax, W, T, post_drift,
                                  fuse && !mixed, next_drift, g.d_status, g.stream);
     rc = launch_error();
     if (rc) return rc;
@@ -760,14 +796,18 @@ int run_substeps(const double *src, double *mid, double *dst, const double *mass
     const int cnt = substeps(order, w, &so);
     const int64_t total = (int64_t)cnt * nsteps;
     const bool fuse = fusable(n);
+    bool prepped = false;
     for (int64_t k = 0; k < total; ++k) {
         const bool last = k == total - 1;
+        const double t = w[k % cnt] * dt;
         const double tn = last ? 0.0 : w[(k + 1) % cnt] * dt;
         const double next_drift = so == 2 ? 0.5 * tn : (so == 1 ? 0.0 : tn);  // as the prep
+        const bool fuse_k = fuse && !last && weak_form(so, t) == weak_form(so, tn);
         const int rc = step_device(k == 0 ? src : mid, last ? dst : mid,
-                                   k == 0 ? masses : step_masses(n), n, w[k % cnt] * dt, so,
-                                   fuse && k > 0, fuse && !last, next_drift);
+                                   k == 0 ? masses : step_masses(n), n, t, so, prepped, fuse_k,
+                                   next_drift);
         if (rc) return rc;
+        prepped = fuse_k;
     }
     return SAKURA_OK;
 }

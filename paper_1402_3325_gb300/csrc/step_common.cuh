@@ -162,7 +162,8 @@ void launch_pair_step_sym(const StepArgs &a, int Smax, int64_t T, int blocks, bo
                           cudaStream_t s);
 // fuse: also apply the next sub-step's drift next_drift and write its
 // drifted copy to X (and X32, if not null), replacing the next prep kernel
-void launch_apply_sym(double *state, double *X, float *X32, const double *partial, int64_t n,
+void launch_apply_sym(double *state, double *X, float *X32, float4 *rows,
+                      const double *partial, int64_t n,
                       int Smax, int64_t W, int64_t T, double post_drift, bool fuse,
                       double next_drift, unsigned *status, cudaStream_t s);
 

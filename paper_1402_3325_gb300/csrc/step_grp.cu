@@ -43,6 +43,7 @@
 #include "pair_batch_fp64.cuh"
 #include "step_common.cuh"
 #include "step_grp.cuh"
+#include "weak_rows.cuh"
 
 namespace sakura {
 
@@ -84,8 +85,8 @@ constexpr int kGrpEmuStandard = kEmuIncMul | kEmuIterMul;
 constexpr int kGrpApplyWarps = 8;
 
 __global__ void __launch_bounds__(32 * kGrpApplyWarps)
-    apply_grp_kernel(double *state, double *X, float *X32, GrpParts parts, int64_t n,
-                     GrpLayout L, int64_t B, double post_drift, int fuse, double next_drift,
+    apply_grp_kernel(double *state, double *X, float *X32, float4 *rows, GrpParts parts,
+                     int64_t n, GrpLayout L, int64_t B, double post_drift, int fuse, double next_drift,
                      unsigned *status)
 {
     __shared__ double red[kGrpApplyWarps][2][32];
@@ -163,18 +164,23 @@ __global__ void __launch_bounds__(32 * kGrpApplyWarps)
             X32[(3 + q) * n + ip] = __double2float_rn(x - (double)hi);
             X32[(6 + q) * n + ip] = __double2float_rn(v1);
         }
+        if (rows) {
+            const double tau = 2.0 * next_drift;
+            weak_row_component(rows, n, ip, q, x1n, v1, tau);
+            if (q == 0) weak_row_mass(rows, n, ip, X[6 * n + ip], tau);
+        }
     }
 }
 
-void launch_apply_grp(double *state, double *X, float *X32, const GrpParts &parts, int64_t n,
-                      const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
+void launch_apply_grp(double *state, double *X, float *X32, float4 *rows, const GrpParts &parts,
+                      int64_t n, const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
                       double next_drift, unsigned *status, cudaStream_t s)
 {
     GrpParts pv = parts;
     GrpLayout Lv = L;
     int64_t B = blocks;
     int f = fuse ? 1 : 0;
-    void *args[] = {(void *)&state,      (void *)&X, (void *)&X32,        (void *)&pv,
+    void *args[] = {(void *)&state,      (void *)&X, (void *)&X32, (void *)&rows, (void *)&pv,
                     (void *)&n,          (void *)&Lv, (void *)&B,         (void *)&post_drift,
                     (void *)&f,          (void *)&next_drift, (void *)&status};
     launch_pdl((const void *)apply_grp_kernel, dim3((unsigned)((n + 31) / 32), 3),

@@ -23,8 +23,8 @@ int pair_step_grp_mixed_blocks_per_sm(bool stats, bool seed);
 // (next_drift), writing its drifted copy to X (and X32, if not null) as the
 // prep kernel would, so that a run of steps needs no prep kernel after its
 // first
-void launch_apply_grp(double *state, double *X, float *X32, const GrpParts &parts, int64_t n,
-                      const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
+void launch_apply_grp(double *state, double *X, float *X32, float4 *rows, const GrpParts &parts,
+                      int64_t n, const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
                       double next_drift, unsigned *status, cudaStream_t s);
 // the symmetric FP64 pair kernel in row-group phases (a.mlp: learned guess;
 // a.X32: single-precision seed; a.mixed: the mixed form's inline class test,

@@ -28,6 +28,7 @@
 #include "mlp_infer.cuh"
 #include "pair_batch_fp64.cuh"
 #include "step_common.cuh"
+#include "weak_rows.cuh"
 
 namespace sakura {
 
@@ -256,8 +257,8 @@ __global__ void __launch_bounds__(128, MIXED ? 2 : ((SEED || LEARNED) ? 3 : 4))
 constexpr int kApplyWarps = 16;
 
 __global__ void __launch_bounds__(32 * kApplyWarps)
-    apply_sym_kernel(double *state, double *X, float *X32, const double *partial, int64_t n,
-                     int Smax, int64_t W, int64_t T, double post_drift, int fuse,
+    apply_sym_kernel(double *state, double *X, float *X32, float4 *rows, const double *partial,
+                     int64_t n, int Smax, int64_t W, int64_t T, double post_drift, int fuse,
                      double next_drift, unsigned *status)
 {
     __shared__ double red[kApplyWarps][2][32];
@@ -319,6 +320,11 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
             X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
             X32[(6 + q) * n + i] = __double2float_rn(v1);
         }
+        if (rows) {
+            const double tau = 2.0 * next_drift;
+            weak_row_component(rows, n, i, q, x1, v1, tau);
+            if (q == 0) weak_row_mass(rows, n, i, X[6 * n + i], tau);
+        }
     }
 }
 
@@ -377,12 +383,12 @@ void launch_pair_step_sym(const StepArgs &a, int Smax, int64_t T, int blocks, bo
                sym_smem(learned), s);
 }
 
-void launch_apply_sym(double *state, double *X, float *X32, const double *partial, int64_t n,
-                      int Smax, int64_t W, int64_t T, double post_drift, bool fuse,
+void launch_apply_sym(double *state, double *X, float *X32, float4 *rows, const double *partial,
+                      int64_t n, int Smax, int64_t W, int64_t T, double post_drift, bool fuse,
                       double next_drift, unsigned *status, cudaStream_t s)
 {
     int f = fuse ? 1 : 0;
-    void *args[] = {(void *)&state,      (void *)&X, (void *)&X32, (void *)&partial,
+    void *args[] = {(void *)&state,      (void *)&X, (void *)&X32, (void *)&rows, (void *)&partial,
                     (void *)&n,          (void *)&Smax, (void *)&W, (void *)&T,
                     (void *)&post_drift, (void *)&f, (void *)&next_drift, (void *)&status};
     launch_pdl((const void *)apply_sym_kernel, dim3((unsigned)((n + 31) / 32), 3),

@@ -1,0 +1,580 @@
+// step_weak.cu -- the symmetric FP64 step whose weakly perturbed pairs take
+// the short solve of kepler_weak.cuh (the FP64 form with the
+// single-precision seed, order 2), on the systolic tiles of step_sym.cu and
+// in the row-group layout of step_grp.cu.
+//
+// A warp solves a tile in systolic steps: lane l owns row l and at step k
+// holds the pair with column (l + k) mod 32, the column's sums travelling
+// from lane to lane by shuffles.  The lanes whose pair is weak add its
+// increments at once (weak_add).  The others (the strong pairs) go to the
+// warp's queue in shared memory and are solved 32 at a time by the seeded
+// FP64 solver, so that a rare close pair does not make its warp run a
+// 75-instruction FP64 solve for one lane; a step with more than
+// kWeakInline strong lanes solves them at once.
+//
+// Bound: the FP64 pipe (18 FP64 instructions per pair and 16 cycles each)
+// and the issue slots (about 930 instructions per pair) nearly alike: ncu at
+// 4000 bodies, 81 % and 55 % before three FP64 instructions more were taken
+// out.  ms per step: 16384 bodies (black hole) 20.36 -> 5.18 in row groups,
+// 5.12 on tiles; Plummer 1024 0.109 -> 0.044, 2048 0.358 -> 0.106, 4000
+// 1.30 -> 0.352 (the kernels of step_sym.cu and step_grp.cu with the seed
+// before).
+#include <cuda_runtime.h>
+
+#include "kepler_df64.cuh"
+#include "kepler_fp64.cuh"
+#include "kepler_weak.cuh"
+#include "pair_batch_fp64.cuh"
+#include "step_common.cuh"
+#include "step_grp.cuh"
+#include "step_weak.cuh"
+#include "weak_rows.cuh"
+
+namespace sakura {
+
+// Strong lanes of a step that are queued at most: a batch solve of more than
+// 8 lanes in place costs no more than a quarter of one in the queue.
+constexpr int kWeakInline = 8;
+// entries of a warp's queue on tiles: a segment's, and a rest below one batch
+constexpr int kWeakQueue = 32 * kWeakInline + 31;
+
+// FP64 solve of 32 strong pairs (i, j), one per lane, from the drifted state
+// and its float copy; the twelve products m_j d, -m_i d to out[lane]
+__device__ __noinline__ void weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
+                                               double (*out)[12], unsigned *status, int *iters,
+                                               int *fb, int *carried)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t n = a.n;
+    const double *X = a.X;
+    const float *X32 = a.X32;
+    const KeplerParams kp{a.tol, a.max_iter, a.bisection};
+    PairSolve p;
+    double mi = 0.0, mj = 0.0;
+    if (valid) {
+        mi = X[6 * n + i];
+        mj = X[6 * n + j];
+        pair_setup(p, a.tau, mi + mj, X[i] - X[j], X[n + i] - X[n + j],
+                   X[2 * n + i] - X[2 * n + j], X[3 * n + i] - X[3 * n + j],
+                   X[4 * n + i] - X[4 * n + j], X[5 * n + i] - X[5 * n + j], a.pre, -1);
+        float dr[3], dv[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            dr[q] = __fadd_rn(__fsub_rn(X32[q * n + i], X32[q * n + j]),
+                              __fsub_rn(X32[(3 + q) * n + i], X32[(3 + q) * n + j]));
+            dv[q] = __fsub_rn(X32[(6 + q) * n + i], X32[(6 + q) * n + j]);
+        }
+        const K32 o = k32_phase1(dr, dv, X32[9 * n + i] + X32[9 * n + j], a.ptau32, a.t32, 2);
+        if (o.ok && dbits(p.t) == dbits(a.tau) && !p.done) {
+            p.s = f2d(o.s);
+        } else if (!p.done) {
+            p.s = p.t * p.ir0;
+            const double cq = 0.5 * p.s * (p.eta0 * p.ir0);
+            if (magbits(cq) < 0x3fe0000000000000LL) p.s = fma(-cq, p.s, p.s);
+        }
+    } else {
+        p.done = true;
+        p.beta = p.s = 0.0;
+        p.iters = 0;
+        p.status = 0;
+        p.carried = false;
+    }
+    double d[6];
+    fp64_solve_warp<true>(p, valid, a.tau, a.post * a.tau, kp, d, *iters, *fb);
+    if (valid) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            out[lane][q] = mj * d[q];
+            out[lane][6 + q] = -mi * d[q];
+        }
+        *status |= p.status;
+    }
+    *carried = valid && p.carried ? 1 : 0;
+}
+
+// Per-warp state of the weak pair kernels.
+struct WeakWarp {
+    int2 *queue;              // [kWeakQueue] strong pairs: i, j | tag << 24
+    double (*sacc)[32];       // [12][32] sums of the tile's inline strong solves
+    double (*res)[12];        // [32][12] results of a batch of strong solves
+    int tail;
+    unsigned status;
+    long long it_sum, slots, fallbacks, carries;
+    int it_max;
+
+    template <bool STATS>
+    __device__ __forceinline__ void count(int lane, int iters, int fb, int carried)
+    {
+        if (STATS) {
+            it_sum += iters;
+            fallbacks += fb;
+            carries += carried;
+            it_max = max(it_max, iters);
+            const int wmax = __reduce_max_sync(0xffffffffu, iters);
+            if (lane == 0) slots += 32LL * wmax;
+        }
+    }
+
+    template <bool STATS>
+    __device__ __forceinline__ void finish(const StepArgs &a, int lane)
+    {
+        status = __reduce_or_sync(0xffffffffu, status);
+        if (lane == 0 && status) atomicOr(a.status, status);
+        if (STATS) {
+            for (int o = 16; o > 0; o >>= 1) {
+                it_sum += __shfl_xor_sync(0xffffffffu, it_sum, o);
+                slots += __shfl_xor_sync(0xffffffffu, slots, o);
+                fallbacks += __shfl_xor_sync(0xffffffffu, fallbacks, o);
+                carries += __shfl_xor_sync(0xffffffffu, carries, o);
+                it_max = max(it_max, __shfl_xor_sync(0xffffffffu, it_max, o));
+            }
+            if (lane == 0) {
+                atomicAdd(&a.stats[kStatIters], (unsigned long long)it_sum);
+                atomicAdd(&a.stats[kStatSlots], (unsigned long long)slots);
+                atomicAdd(&a.stats[kStatFallbacks], (unsigned long long)fallbacks);
+                atomicAdd(&a.stats[kStatCarries], (unsigned long long)carries);
+                atomicMax(&a.stats[kStatMaxIters], (unsigned long long)it_max);
+            }
+        }
+    }
+};
+
+// Steps k0 .. k1 - 1 of the tile of row block 32 I.. (lane l: row i0 + l)
+// and column block 32 J.. (layout indices; L maps them to particles).
+// Returns the tile's sums of the lane's row in row[0..5] and of column
+// (lane + k1 - 1) mod 32 in col[0..5] (positions, then velocities).
+template <bool STATS>
+__device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws, int n, bool rev,
+                                          int i0, int j0, int k0, int k1, int tag, int lane,
+                                          WeakWarp &s, double row[6], double col[6])
+{
+    const float4 *rows = ws.rows;
+    const bool diag = i0 == j0;
+    const int i = i0 + lane;
+    const bool irow = i < n;
+    const int last = n - 1;
+    const int il = rev ? last - min(i, last) : min(i, last);
+    const WeakParticle A =
+        weak_unpack(rows[il], rows[n + il], rows[2 * n + il], rows[3 * n + il]);
+    const float sa = weak_speed2(A);
+    double vr[3] = {0, 0, 0}, vc[3] = {0, 0, 0};
+    dw er[3], rr[3], ec[3], rc[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) er[q] = rr[q] = ec[q] = rc[q] = dw{0.0f, 0.0f};
+    bool dirty = false;
+    for (int k = k0; k < k1; ++k) {
+        const int c = (lane + k) & 31;
+        const int j = j0 + c;
+        const bool valid = irow && j < n && (!diag || c != lane);
+        const int jl = rev ? last - min(j, last) : min(j, last);
+        const WeakParticle B =
+            weak_unpack(rows[jl], rows[n + jl], rows[2 * n + jl], rows[3 * n + jl]);
+        WeakDiff d;
+        const bool weak = weak_class(A, sa, B, d) && valid;
+        if (weak) weak_add(A, B, d, vr, er, rr, vc, ec, rc);
+        const bool strong = valid && !weak;
+        const unsigned mask = __ballot_sync(0xffffffffu, strong);
+        if (STATS) {
+            const int any = __any_sync(0xffffffffu, weak);
+            s.it_sum += weak ? 1 : 0;
+            s.carries += weak ? 1 : 0;
+            s.it_max = max(s.it_max, weak ? 1 : 0);
+            if (lane == 0 && any) s.slots += 32;
+        }
+        if (mask) {
+            if (__popc(mask) <= kWeakInline) {
+                if (strong)
+                    s.queue[s.tail + __popc(mask & ((1u << lane) - 1u))] =
+                        make_int2(i, j | (tag << 24));
+                s.tail += __popc(mask);
+            } else {
+                if (!dirty) {
+#pragma unroll
+                    for (int q = 0; q < 12; ++q) s.sacc[q][lane] = 0.0;
+                    dirty = true;
+                    __syncwarp();
+                }
+                int iters = 0, fb = 0, car = 0;
+                weak_strong_solve(a, strong, rev ? last - i : i, rev ? last - j : j, s.res,
+                                  &s.status, &iters, &fb, &car);
+                s.count<STATS>(lane, iters, fb, car);
+                if (strong) {
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) {
+                        s.sacc[q][lane] += s.res[lane][q];
+                        if (!diag) s.sacc[6 + q][c] += s.res[lane][6 + q];
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        if (!diag && k + 1 < k1) {
+            const int src = (lane + 1) & 31;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                vc[q] = __shfl_sync(0xffffffffu, vc[q], src);
+                ec[q].h = __shfl_sync(0xffffffffu, ec[q].h, src);
+                ec[q].l = __shfl_sync(0xffffffffu, ec[q].l, src);
+                rc[q].h = __shfl_sync(0xffffffffu, rc[q].h, src);
+                rc[q].l = __shfl_sync(0xffffffffu, rc[q].l, src);
+            }
+        }
+    }
+    const int c = (lane + k1 - 1) & 31;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        row[q] = dw_to_double(rr[q]);
+        row[3 + q] = fma(-ws.inv_t, dw_to_double(er[q]), vr[q]);
+        col[q] = -dw_to_double(rc[q]);
+        col[3 + q] = fma(ws.inv_t, dw_to_double(ec[q]), -vc[q]);
+    }
+    if (dirty) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            row[q] += s.sacc[q][lane];
+            col[q] += s.sacc[6 + q][c];
+        }
+        __syncwarp();
+    }
+}
+
+// Tiles (below 4096 bodies): the partition and slots of step_sym.cu.  A
+// segment's sums are written first; the results of its strong pairs are
+// added to the slots afterwards, by the warp that owns them: batches of 32
+// as the queue fills, and what is left at the block's end with the other
+// warps' rests, packed (a warp of a 1024-body step has one or two strong
+// pairs in all).
+template <bool STATS>
+__global__ void __launch_bounds__(128, 3)
+    pair_step_weak_kernel(StepArgs a, WeakStep ws, int Smax, int64_t T)
+{
+    __shared__ int2 queue[4][kWeakQueue];
+    __shared__ double sacc[4][12][32];
+    __shared__ double res[128][12];
+    __shared__ int cnt[4];
+    griddep_wait();
+    griddep_launch();
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const int64_t n = a.n;
+    const int64_t W = (int64_t)gridDim.x * 4;
+    const int64_t w = (int64_t)blockIdx.x * 4 + wib;
+    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0};
+
+    // adds the results of entries e0 .. e0 + m - 1 of the queue, at
+    // res[r0 ..], to their slots (written before): lane c component c
+    auto add_results = [&](int e0, int m, int r0) {
+        for (int e = 0; e < m; ++e) {
+            const int2 q = s.queue[e0 + e];
+            const int i = q.x, j = q.y & 0xffffff, h = q.y >> 24;
+            const int I = i >> 5, J = j >> 5;
+            if (lane < (I == J ? 6 : 12)) {
+                const int64_t slot = lane < 6 ? (int64_t)J * Smax + h : (int64_t)I * Smax + h;
+                const int c = lane < 6 ? lane : lane - 6;
+                double *dst = a.partial + (slot * 6 + c) * n + (lane < 6 ? i : j);
+                *dst += res[r0 + e][lane];
+            }
+        }
+    };
+
+    const int64_t p1 = (w + 1) * T / W;
+    for (int64_t pos = w * T / W; pos < p1;) {
+        const int64_t tile = pos >> 5;
+        const int k0 = (int)(pos & 31);
+        const int k1 = p1 - pos < 32 - k0 ? k0 + (int)(p1 - pos) : 32;
+        const int h = (int)(w - sym_owner(32 * tile, W, T));
+        pos += k1 - k0;
+        int64_t I, J;
+        sym_tile_of(tile, I, J);
+        double row[6], col[6];
+        weak_tile<STATS>(a, ws, (int)n, false, (int)(32 * I), (int)(32 * J), k0, k1, h, lane, s,
+                         row, col);
+        // row sums of rows i to slot (J, h); column sums to slot (I, h)
+        const int64_t i = 32 * I + lane, j = 32 * J + ((lane + k1 - 1) & 31);
+        if (i < n) {
+            double *dst = a.partial + (J * Smax + h) * 6 * n;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) dst[q * n + i] = row[q];
+        }
+        if (I != J && j < n) {
+            double *dst = a.partial + (I * Smax + h) * 6 * n;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) dst[q * n + j] = col[q];
+        }
+        __syncwarp();
+        while (s.tail >= 32) {
+            s.tail -= 32;
+            const int2 q = s.queue[s.tail + lane];
+            int iters = 0, fb = 0, car = 0;
+            weak_strong_solve(a, true, q.x, q.y & 0xffffff, s.res, &s.status, &iters, &fb, &car);
+            s.count<STATS>(lane, iters, fb, car);
+            __syncwarp();
+            add_results(s.tail, 32, 32 * wib);
+            __syncwarp();
+        }
+    }
+    // the rests of the block's four queues, packed into batches
+    if (lane == 0) cnt[wib] = s.tail;
+    __syncthreads();
+    const int c0 = cnt[0], c1 = c0 + cnt[1], c2 = c1 + cnt[2], tot = c2 + cnt[3];
+    if (32 * wib < tot) {
+        const int e = 32 * wib + lane;
+        const bool v = e < tot;
+        const int o = e < c0 ? 0 : (e < c1 ? 1 : (e < c2 ? 2 : 3));
+        const int b0 = o == 0 ? 0 : (o == 1 ? c0 : (o == 2 ? c1 : c2));
+        const int2 q = v ? queue[o][e - b0] : make_int2(0, 0);
+        int iters = 0, fb = 0, car = 0;
+        weak_strong_solve(a, v, q.x, q.y & 0xffffff, s.res, &s.status, &iters, &fb, &car);
+        s.count<STATS>(lane, iters, fb, car);
+    }
+    __syncthreads();
+    add_results(0, s.tail, wib == 0 ? 0 : (wib == 1 ? c0 : (wib == 2 ? c1 : c2)));
+    s.finish<STATS>(a, lane);
+}
+
+// The row-group layout (grp_layout.cuh), from 4096 bodies: a block of G = 4
+// warps sweeps windows of 2 phases, warp w taking row block w of the group
+// in every phase (a heavy particle's pairs are mostly weak and cost what the
+// others' do, so the row blocks need not rotate over the warps as in
+// step_grp.cu, and a warp keeps one row sum per component instead of G).
+// The column blocks are read through L1, which the small shared memory (58
+// KB per block) leaves room for: with rotating rows (78 KB) the step took
+// 6.11 ms at 16384 bodies, this way 5.18; one block of 12 warps per SM 5.43,
+// two of 6 5.36, four of 3 5.27.
+// The strong pairs of a window are solved together by the block, packed
+// into batches of 32, between the window's barriers; each warp adds its own
+// pairs' results to its own sums in queue order (deterministic).
+constexpr int kWeakGrpWindow = 2;
+constexpr size_t weak_grp_smem()
+{
+    return sizeof(double) * kFp64GrpWarps * 32 *
+               (6 * kWeakGrpWindow + 6 + 12 + 12) +
+           sizeof(int2) * kFp64GrpWarps * (32 * kWeakInline * kWeakGrpWindow);
+}
+
+template <bool STATS>
+__global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
+    pair_step_grp_weak_kernel(StepArgs a, WeakStep ws, GrpLayout L, GrpParts parts)
+{
+    constexpr int G = kFp64GrpWarps;
+    constexpr int WIN = kWeakGrpWindow;
+    // column sums of the window's tiles, row sums of the group, inline sums
+    // and batch results per warp, then the warps' queues
+    extern __shared__ __align__(16) unsigned char gsm[];
+    double(*cs)[WIN][6][32] = reinterpret_cast<double(*)[WIN][6][32]>(gsm);
+    double(*rs)[6][32] = reinterpret_cast<double(*)[6][32]>(cs + G);
+    double(*sacc)[12][32] = reinterpret_cast<double(*)[12][32]>(rs + G);
+    double(*res)[12] = reinterpret_cast<double(*)[12]>(sacc + G);
+    int2(*queue)[32 * kWeakInline * WIN] =
+        reinterpret_cast<int2(*)[32 * kWeakInline * WIN]>(res + 32 * G);
+    __shared__ int cnt[G];
+    griddep_wait();
+    griddep_launch();
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const int tid = threadIdx.x;
+    const int64_t n = a.n;
+    const int64_t nb = L.nb;
+    const int64_t B = gridDim.x;
+    const int64_t b = blockIdx.x;
+    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0};
+
+    GrpPos cur = grp_block_start(L, b, B);
+    __shared__ GrpPos s_end;
+    if (tid == 0) s_end = grp_block_start(L, b + 1, B);
+    for (int e = tid; e < G * 6 * 32; e += G * 32) (&rs[0][0][0])[e] = 0.0;
+    __syncthreads();
+    auto in_range = [&](const GrpPos &p) {
+        const GrpPos e = s_end;
+        return p.g < e.g || (p.g == e.g && (p.t < e.t || (p.t == e.t && p.k < e.k)));
+    };
+    auto window_len = [&](const GrpPos &p) {
+        const GrpPos e = s_end;
+        const int64_t m = p.g < e.g ? nb - p.g * G - p.t : e.t - p.t + (e.k > 0 ? 1 : 0);
+        return (int)(m < WIN ? m : WIN);
+    };
+    int wl = in_range(cur) ? window_len(cur) : 0;
+
+    while (wl > 0) {
+        const int64_t g = cur.g, R = grp_rows(L, g), J0 = g * G + cur.t;
+        const int kfirst = cur.k;
+        const int klast = (g == s_end.g && cur.t + wl - 1 == s_end.t) ? s_end.k : 32;
+        for (int cb = 0; cb < wl; ++cb) {
+            const int64_t t = cur.t + cb;
+            const int r = wib;
+            double row[6] = {0, 0, 0, 0, 0, 0}, col[6] = {0, 0, 0, 0, 0, 0};
+            int c = lane;
+            if (r <= t && r < R) {
+                const int64_t I = g * G + r, Jt = J0 + cb;
+                const int kb = cb == 0 ? kfirst : 0;
+                const int ke = cb == wl - 1 ? klast : 32;
+                weak_tile<STATS>(a, ws, (int)n, L.rev != 0, (int)(32 * I), (int)(32 * Jt), kb, ke,
+                                 cb, lane, s, row, col);
+                c = (lane + ke - 1) & 31;
+                if (I == Jt) {
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) col[q] = 0.0;
+                }
+#pragma unroll
+                for (int q = 0; q < 6; ++q) rs[wib][q][lane] += row[q];
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) cs[wib][cb][q][c] = col[q];
+        }
+        // the window's strong pairs, the warps' queues packed into batches;
+        // each warp adds its own pairs' results to its own sums
+        if (lane == 0) cnt[wib] = s.tail;
+        __syncthreads();
+        int base = 0, tot = 0;
+#pragma unroll
+        for (int w = 0; w < G; ++w) {
+            if (w < wib) base += cnt[w];
+            tot += cnt[w];
+        }
+        for (int r0 = 0; r0 < tot; r0 += 32 * G) {
+            if (r0 + 32 * wib < tot) {
+                const int e = r0 + 32 * wib + lane;
+                const bool v = e < tot;
+                int o = 0, eo = e;
+                while (o + 1 < G && eo >= cnt[o]) eo -= cnt[o++];
+                const int2 q = v ? queue[o][eo] : make_int2(0, 0);
+                int iters = 0, fb = 0, car = 0;
+                weak_strong_solve(a, v, (int)grp_particle(L, n, q.x),
+                                  (int)grp_particle(L, n, q.y & 0xffffff), s.res, &s.status,
+                                  &iters, &fb, &car);
+                s.count<STATS>(lane, iters, fb, car);
+            }
+            __syncthreads();
+            const int m0 = max(base, r0), m1 = min(base + s.tail, r0 + 32 * G);
+            for (int e = m0; e < m1; ++e) {
+                const int2 q = s.queue[e - base];
+                const int i = q.x, j = q.y & 0xffffff, cb = q.y >> 24;
+                if (lane < 6)
+                    rs[wib][lane][i & 31] += res[e - r0][lane];
+                else if (lane < 12 && (i >> 5) != (j >> 5))
+                    cs[wib][cb][lane - 6][j & 31] += res[e - r0][lane];
+            }
+            __syncthreads();
+        }
+        s.tail = 0;
+        GrpPos nxt{g, cur.t + wl, 0};
+        if (nxt.t == nb - g * G) {
+            nxt.g = g + 1;
+            nxt.t = 0;
+        }
+        const int wln = in_range(nxt) ? window_len(nxt) : 0;
+        for (int e = tid; e < wl * 192; e += G * 32) {
+            const int cb = e / 192, rem = e - cb * 192, c = rem & 31, q = rem >> 5;
+            double sum = cs[0][cb][q][c];
+#pragma unroll
+            for (int w = 1; w < G; ++w) sum += cs[w][cb][q][c];
+            if (cb == 0 && kfirst > 0) {
+                parts.colx[(b * 6 + q) * 32 + c] = sum;
+            } else {
+                const int64_t j = 32 * (J0 + cb) + c;
+                if (j < n) parts.col[(g * 6 + q) * n + j] = sum;
+            }
+        }
+        if (nxt.g != g || wln == 0) {
+            const int64_t h = b - grp_owner(grp_phase_x(L, g, 0), B, L);
+            double *dst = parts.row + h * 6 * n;
+            for (int e = tid; e < R * 192; e += G * 32) {
+                const int r = e / 192, rem = e - r * 192, l = rem & 31, q = rem >> 5;
+                const int64_t i = 32 * (g * G + r) + l;
+                if (i < n) dst[q * n + i] = rs[r][q][l];
+                rs[r][q][l] = 0.0;
+            }
+        }
+        __syncthreads();
+        cur = nxt;
+        wl = wln;
+    }
+    s.finish<STATS>(a, lane);
+}
+
+// Eq. 27a (order 2), the drifted state with its float copy for the FP64
+// solves, and the rows of the weak pairs; one thread per particle
+__global__ void prep_weak_kernel(const double *state, const double *mass, double *X, float *X32,
+                                 float4 *rows, int64_t n, double tau, unsigned *status)
+{
+    griddep_launch();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double m = mass[i], drift = 0.5 * tau;
+    if (!(m > 0.0)) atomicOr(status, kStatusMass);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double x0 = state[q * n + i], v = state[(3 + q) * n + i];
+        const double x = fma(v, drift, x0);
+        X[q * n + i] = x;
+        X[(3 + q) * n + i] = v;
+        const float hi = __double2float_rn(x);
+        X32[q * n + i] = hi;
+        X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
+        X32[(6 + q) * n + i] = __double2float_rn(v);
+        weak_row_component(rows, n, i, q, x0, v, tau);
+    }
+    X[6 * n + i] = m;
+    X32[9 * n + i] = __double2float_rn(m);
+    weak_row_mass(rows, n, i, m, tau);
+}
+
+int pair_step_weak_blocks_per_sm(bool stats)
+{
+    const void *fn = stats ? (const void *)pair_step_weak_kernel<true>
+                           : (const void *)pair_step_weak_kernel<false>;
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, 128, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return b > 0 ? b : 1;
+}
+
+void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
+                           bool stats, cudaStream_t s)
+{
+    int Sv = Smax;
+    int64_t it = T;
+    void *args[] = {(void *)&a, (void *)&ws, (void *)&Sv, (void *)&it};
+    launch_pdl(stats ? (const void *)pair_step_weak_kernel<true>
+                     : (const void *)pair_step_weak_kernel<false>,
+               dim3(blocks), dim3(128), args, 0, s);
+}
+
+int pair_step_grp_weak_blocks_per_sm(bool stats)
+{
+    const void *fn = stats ? (const void *)pair_step_grp_weak_kernel<true>
+                           : (const void *)pair_step_grp_weak_kernel<false>;
+    int b = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)weak_grp_smem()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kFp64GrpWarps * 32,
+                                                      weak_grp_smem()) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return b > 0 ? b : 1;
+}
+
+void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
+                               const GrpParts &parts, int blocks, bool stats, cudaStream_t s)
+{
+    const void *fn = stats ? (const void *)pair_step_grp_weak_kernel<true>
+                           : (const void *)pair_step_grp_weak_kernel<false>;
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)weak_grp_smem());
+    GrpLayout Lv = L;
+    GrpParts pv = parts;
+    void *args[] = {(void *)&a, (void *)&ws, (void *)&Lv, (void *)&pv};
+    launch_pdl(fn, dim3(blocks), dim3(kFp64GrpWarps * 32), args, weak_grp_smem(), s);
+}
+
+void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
+                      float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s)
+{
+    const int threads = 64;
+    prep_weak_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
+        state, mass, X, X32, rows, n, tau, status);
+}
+
+}  // namespace sakura

@@ -1,0 +1,26 @@
+// step_weak.cuh -- the pair kernels that solve weakly perturbed pairs with
+// kepler_weak.cuh: launchers.
+#pragma once
+
+#include "step_grp.cuh"
+#include "step_common.cuh"
+
+namespace sakura {
+
+// rows [4][n] of the particles as the weak pair kernels read them
+// (kepler_weak.cuh), written by the prep kernel and the fused apply kernels
+struct WeakStep {
+    float4 *rows;
+    double inv_t;  // 1 / tau
+};
+
+void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
+                      float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s);
+void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
+                           bool stats, cudaStream_t s);
+int pair_step_weak_blocks_per_sm(bool stats);
+void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
+                               const GrpParts &parts, int blocks, bool stats, cudaStream_t s);
+int pair_step_grp_weak_blocks_per_sm(bool stats);
+
+}  // namespace sakura

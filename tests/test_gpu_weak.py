@@ -1,0 +1,83 @@
+"""The seeded FP64 step's weak pairs (csrc/kepler_weak.cuh, csrc/step_weak.cu)
+on tiles and in row groups against the oracle, at ragged sizes and for mixes
+of weak and strong pairs."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1402_3325_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12  # as tests/test_gpu_step.py
+NCPU = os.cpu_count() or 1
+
+
+def _step(s, dt, order=2, nsteps=1, **options):
+    import torch
+    from paper_1402_3325_gb300 import sakura as sk
+    sk.init(0, stream=torch.cuda.current_stream().cuda_stream, guess=sk.GUESS_FP32, **options)
+    state = torch.tensor(s.soa(), device="cuda")
+    mass = torch.tensor(s.m, device="cuda")
+    sk.get_stats(reset=True)
+    if nsteps == 1:
+        sk.step(state, mass, dt, order)
+    else:
+        sk.evolve(state, mass, dt, order, nsteps)
+    sk.check()
+    return ics.from_soa(state.cpu().numpy()), sk.get_stats(reset=True)
+
+
+def _close(got, ref, tol=TOL):
+    for a, b in zip(got, ref):
+        scale = np.maximum(np.linalg.norm(b, axis=1), np.sqrt((b ** 2).sum(1).mean()))
+        assert (np.linalg.norm(a - b, axis=1) <= tol * scale).all()
+
+
+def _kinds(n):
+    yield "cluster", ics.random_cluster(n, seed=n, mass_spread=3.0)
+    s = ics.random_cluster(n, seed=n + 1)       # in a plane: exact zero differences
+    s.r[:, 2] = s.v[:, 2] = 0.0
+    yield "planar", s
+    if n < 1000:                                # fast: every pair strong (at 1000 bodies the
+        s = ics.random_cluster(n, seed=n + 2)   # map amplifies any rounding to 1e-9)
+        yield "swarm", ics.System(s.m, s.r * 1e-3, s.v * 100.0, s.dt)
+    s = ics.random_cluster(n, seed=n + 3)       # separations of exact powers of two
+    s.r[:, :] = np.stack(np.unravel_index(np.arange(n), (16, 16, 32)), 1) * 2.0 ** -2
+    yield "lattice", s
+
+
+@pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("n", [21, 32, 33, 64, 95, 129, 1000])
+def test_weak_step_matches_oracle(n, flag):
+    for name, s in _kinds(n):
+        got, st = _step(s, s.dt, flags=flag | 2)
+        rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
+        assert rc == oracle.OK
+        _close(got, (r, v))
+        assert st["iters"] >= st["solves"]
+        again, _ = _step(s, s.dt, flags=flag | 2)
+        assert np.array_equal(got[0], again[0]) and np.array_equal(got[1], again[1])
+        if name == "planar":
+            assert not got[0][:, 2].any() and not got[1][:, 2].any()
+
+
+@pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("blocks", [1, 5, 151, 4000])
+def test_weak_step_on_any_grid(flag, blocks):
+    s = ics.plummer_binaries(700, seed=4)
+    s = ics.System(s.m, s.r, s.v, 2.0 ** -7)  # a few per cent of strong pairs
+    got, _ = _step(s, s.dt, flags=flag, grid_blocks=blocks)
+    rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
+    _close(got, (r, v))
+
+
+@pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("order,dt", [(4, 2.0 ** -8), (2, -(2.0 ** -8)), (2, 1e-17), (2, 1e-19),
+                                      (2, 0.0), (2, 2.0)])
+def test_weak_step_orders_and_step_sizes(flag, order, dt):
+    s = ics.random_cluster(150, seed=8)
+    got, _ = _step(s, dt, order, 3, flags=flag)
+    rc, r, v = oracle.evolve(s.m, s.r, s.v, dt, 3, order, nthreads=NCPU)
+    _close(got, (r, v), 1e-10 if dt == 2.0 else 12 * TOL)
