@@ -4,12 +4,12 @@
 // is run with the FP64 solver (standard guess) and the features of
 // mlp_infer.cuh and the target g = log(s / s_T2) / w are written.
 //
-// Training (FP32, the project's own kernels):
-//   forward/backward kernel: one thread per sample computes the forward pass,
-//     the residual and the back-propagated dz2, dz1 (stored per sample);
-//   gradient kernels: each weight gradient is a sum over the batch, computed
-//     by one thread per weight in sample order (deterministic, no atomics);
-//   Adam kernel: bias-corrected Adam update of the FP32 master parameters.
+// Training (FP32, the project's own kernels), two launches per minibatch:
+//   tile kernel: forward and backward pass of 32 samples per block and the
+//     block's sums of every gradient;
+//   reduce kernel: the blocks' sums added in a fixed order (deterministic, no
+//     atomics), then the gradient written or the bias-corrected Adam update
+//     of the FP32 master parameters.
 // Parameter layout (FP32): W1[64][6], b1[64], W2[64][64], b2[64], W3[64], b3.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -74,92 +74,256 @@ __global__ void __launch_bounds__(128)
 }
 
 // ------------------------------------------------------------- training
-// dy, dz2 [B][64], dz1 [B][64], h1, h2 [B][64], xn [B][6], r2 (squared
-// residuals) are per-sample scratch.
-__global__ void __launch_bounds__(64)
-    mlp_fwd_bwd_kernel(const float *P, const float *norm, const float *feat, const float *target,
-                       int64_t B, float *xn, float *h1, float *h2, float *dy, float *dz2,
-                       float *dz1, float *r2)
+// Forward and backward pass of 32 samples at a time, with the tile's
+// contribution to every gradient kept in the block's registers until the
+// block's last tile; partial [gridDim.x][kMlpGradStride] receives each
+// block's sums (the 4673 gradients, then the squared residuals).
+//
+// Bound: the three 32 x 64 x 64 products of a tile on the FP32 pipe, fed from
+// shared memory.  A thread forms 2 x 4 (or 4 x 4) outputs and reads its
+// operands as float4 along the summed index, so 6 (8) loads serve 32 (64)
+// FMAs; rows are padded to 68 (36) floats, which spreads the 16 rows that a
+// warp reads over the banks.  Each pre-activation is one chain of FMAs in
+// ascending k from the bias.
+// The kernels before took one thread per sample (activations in local memory
+// and per-sample arrays in global memory) and one thread per weight walking
+// the batch: 455 us per minibatch of 8192, the sums over the batch in
+// one chain of 8192 roundings.
+constexpr int kMlpTile = 32, kMlpThreads = 256;
+constexpr int kMlpRow = 68, kMlpCol = 36;  // padded row lengths
+constexpr int kMlpGradStride = 4736;       // floats of a block's sums, 4674 used
+
+struct MlpSmem {
+    float W2[64 * kMlpRow], W2T[64 * kMlpRow];           // [o][k], [k][o]
+    float hS[kMlpTile * kMlpRow], dS[kMlpTile * kMlpRow];  // [s][k]: h1; h2, then dz2
+    float hT[64 * kMlpCol], dT[64 * kMlpCol];            // [k][s]: h1; dz2, then dz1
+    float x[kMlpTile * 8], W1[64 * 8], W3[64], b1[64], b2[64], g[kMlpTile], r2[kMlpTile];
+};
+
+__device__ __forceinline__ float dot4(float4 a, float4 b, float c)
 {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    float x[6];
-    for (int k = 0; k < 6; ++k) {
-        x[k] = (feat[b * 6 + k] - norm[k]) / norm[6 + k];
-        xn[b * 6 + k] = x[k];
-    }
-    float a1[64];
-    for (int o = 0; o < 64; ++o) {
-        float z = P[kOffB1 + o];
-        for (int k = 0; k < 6; ++k) z = fmaf(P[kOffW1 + o * 6 + k], x[k], z);
-        a1[o] = tanhf(z);
-        h1[b * 64 + o] = a1[o];
-    }
-    float y = P[kOffB3];
-    for (int o = 0; o < 64; ++o) {
-        float z = P[kOffB2 + o];
-        for (int k = 0; k < 64; ++k) z = fmaf(P[kOffW2 + o * 64 + k], a1[k], z);
-        const float a2 = tanhf(z);
-        h2[b * 64 + o] = a2;
-        y = fmaf(P[kOffW3 + o], a2, y);
-    }
-    const float r = y - target[b];
-    r2[b] = r * r;
-    const float g = 2.0f * r / (float)B;
-    dy[b] = g;
-    float dh1[64];
-    for (int k = 0; k < 64; ++k) dh1[k] = 0.0f;
-    for (int o = 0; o < 64; ++o) {
-        const float a2 = h2[b * 64 + o];
-        const float d2 = g * P[kOffW3 + o] * (1.0f - a2 * a2);
-        dz2[b * 64 + o] = d2;
-        for (int k = 0; k < 64; ++k) dh1[k] = fmaf(P[kOffW2 + o * 64 + k], d2, dh1[k]);
-    }
-    for (int k = 0; k < 64; ++k) dz1[b * 64 + k] = dh1[k] * (1.0f - a1[k] * a1[k]);
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
 }
 
-// grad[p] = sum_b left[b][row(p)] * right[b][col(p)] for each weight, plus
-// bias gradients and the loss.  One thread per gradient entry.
-__global__ void mlp_grad_kernel(const float *xn, const float *h1, const float *h2,
-                                const float *dy, const float *dz2, const float *dz1,
-                                const float *r2, int64_t B, float *grad, float *loss)
+__global__ void __launch_bounds__(kMlpThreads)
+    mlp_tile_kernel(const float *P, const float *norm, const float *feat, const float *target,
+                    int64_t B, float *partial)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kMlpParams) return;
-    float acc = 0.0f;
-    if (p < kOffB1) {  // W1[o][k]
-        const int o = p / 6, k = p % 6;
-        for (int64_t b = 0; b < B; ++b) acc = fmaf(dz1[b * 64 + o], xn[b * 6 + k], acc);
-    } else if (p < kOffW2) {
-        const int o = p - kOffB1;
-        for (int64_t b = 0; b < B; ++b) acc += dz1[b * 64 + o];
-    } else if (p < kOffB2) {  // W2[o][k]
-        const int q = p - kOffW2, o = q / 64, k = q % 64;
-        for (int64_t b = 0; b < B; ++b) acc = fmaf(dz2[b * 64 + o], h1[b * 64 + k], acc);
-    } else if (p < kOffW3) {
-        const int o = p - kOffB2;
-        for (int64_t b = 0; b < B; ++b) acc += dz2[b * 64 + o];
-    } else if (p < kOffB3) {
-        const int o = p - kOffW3;
-        for (int64_t b = 0; b < B; ++b) acc = fmaf(dy[b], h2[b * 64 + o], acc);
-    } else if (p == kOffB3) {
-        for (int64_t b = 0; b < B; ++b) acc += dy[b];
-    } else {  // p == kMlpParams: the loss
-        for (int64_t b = 0; b < B; ++b) acc += r2[b];
-        acc /= (float)B;
-        *loss = acc;
+    extern __shared__ __align__(16) unsigned char msm[];
+    MlpSmem &sm = *reinterpret_cast<MlpSmem *>(msm);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    griddep_wait();    // P from the update before, partial read by it
+    griddep_launch();
+    for (int e = tid; e < 4096; e += kMlpThreads) {
+        const float w = P[kOffW2 + e];
+        sm.W2[(e >> 6) * kMlpRow + (e & 63)] = w;
+        sm.W2T[(e & 63) * kMlpRow + (e >> 6)] = w;
+    }
+    for (int e = tid; e < 384; e += kMlpThreads) sm.W1[(e / 6) * 8 + e % 6] = P[kOffW1 + e];
+    if (tid < 64) {
+        sm.W3[tid] = P[kOffW3 + tid];
+        sm.b1[tid] = P[kOffB1 + tid];
+        sm.b2[tid] = P[kOffB2 + tid];
+    }
+    const float b3 = P[kOffB3];
+    // gradient sums: W2[ty + 16 i][tx + 16 j]; of the entries of one weight
+    // or bias, thread tid's
+    float gW2[4][4] = {}, gW1[2] = {0.0f, 0.0f}, gb = 0.0f, gW3 = 0.0f, gb3 = 0.0f, loss = 0.0f;
+    for (int64_t t0 = (int64_t)blockIdx.x * kMlpTile; t0 < B;
+         t0 += (int64_t)gridDim.x * kMlpTile) {
+        __syncthreads();  // the weights; the previous tile's readers
+        for (int e = tid; e < kMlpTile * 6; e += kMlpThreads) {
+            const int s = e / 6, k = e - 6 * s;
+            sm.x[s * 8 + k] = t0 + s < B ? (feat[t0 * 6 + e] - norm[k]) / norm[6 + k] : 0.0f;
+        }
+        __syncthreads();
+        // h1: 8 units of one sample per thread
+        {
+            const int s = tid >> 3;
+            for (int o = tid & 7; o < 64; o += 8) {
+                float z = sm.b1[o];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) z = fmaf(sm.W1[o * 8 + k], sm.x[s * 8 + k], z);
+                const float h = tanhf(z);
+                sm.hS[s * kMlpRow + o] = h;
+                sm.hT[o * kMlpCol + s] = h;
+            }
+        }
+        __syncthreads();
+        // h2 of samples 2 ty, 2 ty + 1 and units tx + 16 i
+        float z[2][4], h2[2][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[0][i] = z[1][i] = sm.b2[tx + 16 * i];
+#pragma unroll 4
+        for (int k = 0; k < 64; k += 4) {
+            const float4 a0 = *(const float4 *)&sm.hS[(2 * ty) * kMlpRow + k];
+            const float4 a1 = *(const float4 *)&sm.hS[(2 * ty + 1) * kMlpRow + k];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 w = *(const float4 *)&sm.W2[(tx + 16 * i) * kMlpRow + k];
+                z[0][i] = dot4(w, a0, z[0][i]);
+                z[1][i] = dot4(w, a1, z[1][i]);
+            }
+        }
+        // y, the residual and dy: the 16 lanes of a half warp hold one sample's units
+        float y[2] = {0.0f, 0.0f};
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                h2[u][i] = tanhf(z[u][i]);
+                y[u] = fmaf(sm.W3[tx + 16 * i], h2[u][i], y[u]);
+                sm.dS[(2 * ty + u) * kMlpRow + tx + 16 * i] = h2[u][i];
+            }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            y[0] += __shfl_xor_sync(0xffffffffu, y[0], o);
+            y[1] += __shfl_xor_sync(0xffffffffu, y[1], o);
+        }
+        float dy[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t b = t0 + 2 * ty + u;
+            const float r = b < B ? y[u] + b3 - target[b] : 0.0f;
+            dy[u] = 2.0f * r / (float)B;
+            if (tx == 0) {
+                sm.g[2 * ty + u] = dy[u];
+                sm.r2[2 * ty + u] = r * r;
+            }
+        }
+        __syncthreads();
+        // dW3 (64 threads), db3 and the loss (one warp)
+        if (tid < 64) {
+            for (int s = 0; s < kMlpTile; ++s)
+                gW3 = fmaf(sm.g[s], sm.dS[s * kMlpRow + tid], gW3);
+        } else if (tid < 96) {
+            gb3 += sm.g[tid - 64];
+            loss += sm.r2[tid - 64];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int o = tx + 16 * i;
+                const float d2 = dy[u] * sm.W3[o] * (1.0f - h2[u][i] * h2[u][i]);
+                sm.dS[(2 * ty + u) * kMlpRow + o] = d2;
+                sm.dT[o * kMlpCol + 2 * ty + u] = d2;
+            }
+        __syncthreads();
+        // dW2[ty + 16 i][tx + 16 j], db2
+#pragma unroll 2
+        for (int s = 0; s < kMlpTile; s += 4) {
+            float4 a[4], h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = *(const float4 *)&sm.dT[(ty + 16 * i) * kMlpCol + s];
+                h[i] = *(const float4 *)&sm.hT[(tx + 16 * i) * kMlpCol + s];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) gW2[i][j] = dot4(a[i], h[j], gW2[i][j]);
+        }
+        if (tid >= 64 && tid < 128)
+            for (int s = 0; s < kMlpTile; ++s) gb += sm.dT[(tid - 64) * kMlpCol + s];
+        // dh1 of samples 2 ty, 2 ty + 1 and units tx + 16 i
+        float d1[2][4] = {};
+#pragma unroll 4
+        for (int o = 0; o < 64; o += 4) {
+            const float4 a0 = *(const float4 *)&sm.dS[(2 * ty) * kMlpRow + o];
+            const float4 a1 = *(const float4 *)&sm.dS[(2 * ty + 1) * kMlpRow + o];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 w = *(const float4 *)&sm.W2T[(tx + 16 * i) * kMlpRow + o];
+                d1[0][i] = dot4(w, a0, d1[0][i]);
+                d1[1][i] = dot4(w, a1, d1[1][i]);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int k = tx + 16 * i;
+                const float h = sm.hS[(2 * ty + u) * kMlpRow + k];
+                sm.dT[k * kMlpCol + 2 * ty + u] = d1[u][i] * (1.0f - h * h);
+            }
+        __syncthreads();
+        // dW1 (entries tid and 256 + tid), db1
+        if (tid < 64)
+            for (int s = 0; s < kMlpTile; ++s) gb += sm.dT[tid * kMlpCol + s];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = tid + 256 * q;
+            if (e < 384)
+                for (int s = 0; s < kMlpTile; ++s)
+                    gW1[q] = fmaf(sm.dT[(e / 6) * kMlpCol + s], sm.x[s * 8 + e % 6], gW1[q]);
+        }
+    }
+    float *out = partial + (int64_t)blockIdx.x * kMlpGradStride;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[kOffW2 + (ty + 16 * i) * 64 + tx + 16 * j] = gW2[i][j];
+    out[kOffW1 + tid] = gW1[0];
+    if (tid + 256 < 384) out[kOffW1 + tid + 256] = gW1[1];
+    if (tid < 64) {
+        out[kOffB1 + tid] = gb;
+        out[kOffW3 + tid] = gW3;
+    } else if (tid < 128) {
+        out[kOffB2 + tid - 64] = gb;
+    }
+    if (tid >= 64 && tid < 96) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+            loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        }
+        if (tid == 64) {
+            out[kOffB3] = gb3;
+            out[kMlpParams] = loss;
+        }
+    }
+}
+
+// Sums of the blocks' gradients: 32 entries per block of 256 threads, each
+// of its 8 warps taking every eighth partial, the warps' sums added in warp
+// order.  Then either the gradient is written (grad) or, in training, one
+// Adam step taken (m, v; bias corrections 1 - b1t, 1 - b2t).
+__global__ void __launch_bounds__(256)
+    mlp_reduce_kernel(const float *partial, int blocks, int64_t B, float *grad, float *loss,
+                      float *P, float *m, float *v, float lr, float b1t, float b2t)
+{
+    __shared__ float red[8][32];
+    griddep_wait();
+    griddep_launch();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    float s0 = 0.0f, s1 = 0.0f;
+    if (p <= kMlpParams) {
+        int b = w;
+        for (; b + 8 < blocks; b += 16) {
+            s0 += partial[(int64_t)b * kMlpGradStride + p];
+            s1 += partial[(int64_t)(b + 8) * kMlpGradStride + p];
+        }
+        if (b < blocks) s0 += partial[(int64_t)b * kMlpGradStride + p];
+    }
+    red[w][lane] = s0 + s1;
+    __syncthreads();
+    if (w != 0 || p > kMlpParams) return;
+    float gi = red[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) gi += red[k][lane];
+    if (p == kMlpParams) {
+        *loss = gi / (float)B;
         return;
     }
-    grad[p] = acc;
-}
-
-__global__ void adam_kernel(float *P, float *m, float *v, const float *g, int n, float lr,
-                            float b1t, float b2t)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+    if (grad) {
+        grad[p] = gi;
+        return;
+    }
     const float b1 = 0.9f, b2 = 0.999f;
-    const float gi = g[p];
     const float mi = b1 * m[p] + (1.0f - b1) * gi;
     const float vi = b2 * v[p] + (1.0f - b2) * gi * gi;
     m[p] = mi;
@@ -224,29 +388,39 @@ void launch_sample_pairs(const double *X, int64_t n, double tau, double pre, con
                                                          iters, tol, status);
 }
 
-void launch_mlp_grad(const float *P, const float *norm, const float *feat, const float *target,
-                     int64_t B, float *scratch, float *grad, float *loss, cudaStream_t s)
+namespace {
+
+// one tile of 32 samples per block, up to two blocks' worth per SM (a block's
+// sums are 19 KB of scratch)
+int mlp_blocks(int64_t B)
 {
-    float *xn = scratch;
-    float *h1 = xn + B * 6;
-    float *h2 = h1 + B * 64;
-    float *dz2 = h2 + B * 64;
-    float *dz1 = dz2 + B * 64;
-    float *dy = dz1 + B * 64;
-    float *r2 = dy + B;
-    mlp_fwd_bwd_kernel<<<(unsigned)((B + 63) / 64), 64, 0, s>>>(P, norm, feat, target, B, xn, h1,
-                                                                h2, dy, dz2, dz1, r2);
-    mlp_grad_kernel<<<(kMlpParams + 1 + 127) / 128, 128, 0, s>>>(xn, h1, h2, dy, dz2, dz1, r2, B,
-                                                                 grad, loss);
+    const int64_t tiles = (B + kMlpTile - 1) / kMlpTile;
+    return (int)(tiles < 304 ? tiles : 304);
 }
 
-size_t mlp_grad_scratch_floats(int64_t B) { return (size_t)B * (6 + 64 * 4 + 2); }
+}  // namespace
 
-void launch_adam(float *P, float *m, float *v, const float *g, float lr, float b1t, float b2t,
-                 cudaStream_t s)
+void launch_mlp_step(float *P, const float *norm, const float *feat, const float *target,
+                     int64_t B, float *scratch, float *grad, float *loss, float *m, float *v,
+                     float lr, float b1t, float b2t, cudaStream_t s)
 {
-    adam_kernel<<<(kMlpParams + 127) / 128, 128, 0, s>>>(P, m, v, g, kMlpParams, lr, b1t, b2t);
+    int blocks = mlp_blocks(B);
+    const size_t smem = sizeof(MlpSmem);
+    cudaFuncSetAttribute((const void *)mlp_tile_kernel,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const float *Pc = P;
+    void *a1[] = {(void *)&Pc, (void *)&norm, (void *)&feat, (void *)&target, (void *)&B,
+                  (void *)&scratch};
+    launch_pdl((const void *)mlp_tile_kernel, dim3(blocks), dim3(kMlpThreads), a1, smem, s);
+    const float *part = scratch;
+    void *a2[] = {(void *)&part, (void *)&blocks, (void *)&B, (void *)&grad, (void *)&loss,
+                  (void *)&P,    (void *)&m,      (void *)&v, (void *)&lr,   (void *)&b1t,
+                  (void *)&b2t};
+    launch_pdl((const void *)mlp_reduce_kernel, dim3((kMlpParams + 1 + 31) / 32), dim3(256), a2, 0,
+               s);
 }
+
+size_t mlp_grad_scratch_floats(int64_t B) { return (size_t)mlp_blocks(B) * kMlpGradStride; }
 
 void launch_mlp_pack(const float *blob, MlpWeights *W, cudaStream_t s)
 {

@@ -1366,8 +1366,9 @@ int sakura_mlp_grad(const float *params, const float *norm, const float *feature
         return SAKURA_E_ARG;
     int rc = grow(g.mlp_scratch, sakura::mlp_grad_scratch_floats(batch) * sizeof(float));
     if (rc) return rc;
-    sakura::launch_mlp_grad(params, norm, features, targets, batch, (float *)g.mlp_scratch.ptr,
-                            grad, loss, g.stream);
+    sakura::launch_mlp_step(const_cast<float *>(params), norm, features, targets, batch,
+                            (float *)g.mlp_scratch.ptr, grad, loss, nullptr, nullptr, 0.0f, 0.0f,
+                            0.0f, g.stream);
     if (launch_error()) return SAKURA_E_CUDA;
     return cudaStreamSynchronize(g.stream) == cudaSuccess ? SAKURA_OK : SAKURA_E_CUDA;
 }
@@ -1384,8 +1385,8 @@ int sakura_mlp_train(float *params, const float *norm, const float *features,
     const int P = sakura::kMlpParams;
     int rc = grow(g.mlp_scratch, sakura::mlp_grad_scratch_floats(batch) * sizeof(float));
     if (rc) return rc;
-    if ((rc = grow(g.mlp_adam, (size_t)(3 * P + 1) * sizeof(float)))) return rc;
-    float *m = (float *)g.mlp_adam.ptr, *v = m + P, *gr = v + P, *lossbuf = gr + P;
+    if ((rc = grow(g.mlp_adam, (size_t)(2 * P + 1) * sizeof(float)))) return rc;
+    float *m = (float *)g.mlp_adam.ptr, *v = m + P, *lossbuf = v + P;
     if (cudaMemsetAsync(m, 0, 2 * P * sizeof(float), g.stream) != cudaSuccess)
         return SAKURA_E_CUDA;
     const int64_t per_epoch = nsamples / batch;
@@ -1395,12 +1396,12 @@ int sakura_mlp_train(float *params, const float *norm, const float *features,
         for (int64_t k = 0; k < per_epoch; ++k) {
             const int64_t off = k * batch;
             float *lp = losses ? losses + t : lossbuf;
-            sakura::launch_mlp_grad(params, norm, features + off * 6, targets + off, batch,
-                                    (float *)g.mlp_scratch.ptr, gr, lp, g.stream);
             ++t;
             b1t *= 0.9;
             b2t *= 0.999;
-            sakura::launch_adam(params, m, v, gr, lr, (float)b1t, (float)b2t, g.stream);
+            sakura::launch_mlp_step(params, norm, features + off * 6, targets + off, batch,
+                                    (float *)g.mlp_scratch.ptr, nullptr, lp, m, v, lr, (float)b1t,
+                                    (float)b2t, g.stream);
         }
     }
     if (launch_error()) return SAKURA_E_CUDA;

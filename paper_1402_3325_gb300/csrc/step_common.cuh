@@ -147,11 +147,12 @@ int pair_step_fp64_blocks_per_sm(int warps, bool stats, bool learned = false);
 void launch_sample_pairs(const double *X, int64_t n, double tau, double pre, const int64_t *ids,
                          int64_t count, float *feat, float *target, int *iters, double tol,
                          unsigned *status, cudaStream_t s);
-void launch_mlp_grad(const float *P, const float *norm, const float *feat, const float *target,
-                     int64_t B, float *scratch, float *grad, float *loss, cudaStream_t s);
+// one minibatch: the gradient and loss (grad), or one Adam step of P (grad
+// null: moments m and v, bias corrections 1 - b1t, 1 - b2t) and the loss
+void launch_mlp_step(float *P, const float *norm, const float *feat, const float *target,
+                     int64_t B, float *scratch, float *grad, float *loss, float *m, float *v,
+                     float lr, float b1t, float b2t, cudaStream_t s);
 size_t mlp_grad_scratch_floats(int64_t B);
-void launch_adam(float *P, float *m, float *v, const float *g, float lr, float b1t, float b2t,
-                 cudaStream_t s);
 void launch_mlp_pack(const float *blob, MlpWeights *W, cudaStream_t s);
 void launch_mlp_eval(const MlpWeights *W, const float *feat, int64_t count, float *out,
                      cudaStream_t s);
