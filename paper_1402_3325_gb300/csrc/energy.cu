@@ -1,22 +1,33 @@
 // energy.cu -- total energy E = T + U of a device state (Eqs. 1-3).
 //
-// Stage 1: each warp takes row pairs (i, n-1-i) so that every warp sees the
-// same number of pair terms, lanes stride over j > i, and every lane keeps a
-// double-double (two-sum) accumulator of -m_i m_j / r_ij.  Warps reduce their
-// lanes in double-double and write one (hi, lo) pair each.
+// Stage 1: rows r and n-1-r have n - 1 pairs (j > i) between them; the list
+// of these row pairs, each cut into S equal segments, is dealt to the warps,
+// lanes stride over j.  A lane sums m_j / r_ij of four pairs and adds the sum
+// to a double-double (Fast2Sum, Dekker 1971, of the operands in order of
+// size); the row's factor -m_i is applied once per row, in double-double.
+// Warps reduce their lanes in double-double and write one (hi, lo) pair each.
 // Stage 2: one block adds the kinetic terms m_i v_i^2 / 2 and the warp
-// partials in a fixed order, in double-double.  No atomics on FP64 data; the
-// result does not depend on timing.
+// partials in a fixed order, in double-double, and writes E and the status
+// word to page-locked host memory (a copy-engine read costs about 10 us more
+// per call).  No atomics on FP64 data; the result does not depend on timing.
+//
+// Bound: the FP64 pipe, 10.5 instructions per pair at 16 cycles per warp
+// instruction and SM (2.4 ms at 16384 bodies).  1/r comes from a
+// single-precision value y by one Newton step in FP64, 1/r = y (1 + e/2 +
+// 3 e^2/8), e = 1 - r^2 y^2 with y^2 exact on the integer pipe; the last
+// term, below 2^-43 of the value, is summed in single precision.  With sqrt,
+// a division and a six-operation TwoSum per pair it took 7.96 ms.
 #include <cuda_runtime.h>
 
 #include "kepler_fp64.cuh"
+#include "kepler_weak.cuh"
 #include "step_common.cuh"
 
 namespace sakura {
 namespace {
 
 constexpr int kEnergyThreads = 256;
-constexpr int kEnergyBlocks = 152 * 4;
+constexpr int kEnergyBlocks = 152 * 3;
 
 __device__ __forceinline__ void dd_add(double &s, double &c, double x)
 {
@@ -33,21 +44,66 @@ __device__ __forceinline__ void dd_merge(double &s, double &c, double s2, double
     c += c2;
 }
 
-__device__ __forceinline__ void row_potential(const double *state, const double *mass, int64_t n,
-                                              int64_t i, int lane, double &s, double &c,
-                                              unsigned &st)
+// s + c += x, c the sum of the rounding errors
+__device__ __forceinline__ void dd_add_ordered(double &s, double &c, double x)
 {
-    const double xi = state[i], yi = state[n + i], zi = state[2 * n + i], mi = mass[i];
-    for (int64_t j = i + 1 + lane; j < n; j += 32) {
-        const double dx = xi - state[j], dy = yi - state[n + j], dz = zi - state[2 * n + j];
-        const double d = sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
-        if (!(d > 0.0)) st |= kStatusCoincident;
-        dd_add(s, c, -(mi * mass[j]) / d);
-    }
+    const bool swap = magbits(x) > magbits(s);
+    const double big = swap ? x : s, sml = swap ? s : x;
+    s = big + sml;
+    c += sml - (s - big);
 }
 
-__global__ void __launch_bounds__(kEnergyThreads)
-    energy_pairs_kernel(const double *state, const double *mass, int64_t n, double *work,
+// m / sqrt(r2); the term below 2^-43 of it goes to lo, in single precision,
+// where the value is in float's range
+__device__ __forceinline__ double inv_distance(double r2, double m, float &lo)
+{
+    const long long b = dbits(r2);
+    // outside [2^-120, 2^120): zero (reported by the caller), subnormal,
+    // overflown or not a number
+    if (!((unsigned long long)b - 0x3870000000000000ULL < 0x0f00000000000000ULL))
+        return m / sqrt(r2);
+    const float y = rsqrt_approx(trunc_to_f32(b));
+    // e / 2 = 1/2 - (r2 / 2) y^2
+    const double eh = fma(-__longlong_as_double(b - (1LL << 52)), square_exact(y), 0.5);
+    const double t = m * widen_f32(y);
+    const long long bt = dbits(t), be = dbits(eh);
+    if ((bt & kInfBits) - 0x39b0000000000000LL < 0x0c80000000000000LL &&
+        (bt & kInfBits) >= 0x39b0000000000000LL) {  // 2^-100 <= |t| < 2^100
+        const float ef = (be & kInfBits) >= 0x39b0000000000000LL ? trunc_to_f32(be) : 0.0f;
+        lo = fmaf(1.5f * ef * ef, trunc_to_f32(bt), lo);
+        return fma(t, eh, t);
+    }
+    return fma(t, fma(1.5 * eh, eh, eh), t);
+}
+
+// -m_i sum_j m_j / r_ij over j0 <= j < j1 (this lane's), added to (s, c)
+__device__ __forceinline__ void row_potential(const double *state, const double *mass, int64_t n,
+                                              int64_t i, int64_t j0, int64_t j1, int lane,
+                                              double &s, double &c, unsigned &st)
+{
+    const double xi = state[i], yi = state[n + i], zi = state[2 * n + i], mi = mass[i];
+    double us = 0.0, uc = 0.0;
+    float lo = 0.0f;
+    auto term = [&](int64_t j) {
+        const double dx = xi - state[j], dy = yi - state[n + j], dz = zi - state[2 * n + j];
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        if (!(dbits(r2) > 0 && dbits(r2) <= kInfBits)) st |= kStatusCoincident;
+        return inv_distance(r2, mass[j], lo);
+    };
+    int64_t j = j0 + lane;
+    for (; j + 96 < j1; j += 128) {
+        const double a = term(j), b = term(j + 32), d = term(j + 64), e = term(j + 96);
+        dd_add_ordered(us, uc, (a + b) + (d + e));
+    }
+    for (; j < j1; j += 32) dd_add_ordered(us, uc, term(j));
+    uc += (double)lo;
+    const double p = -mi * us;
+    dd_add(s, c, p);
+    c += fma(-mi, us, -p) - mi * uc;
+}
+
+__global__ void __launch_bounds__(kEnergyThreads, 3)
+    energy_pairs_kernel(const double *state, const double *mass, int64_t n, int S, double *work,
                         unsigned *status)
 {
     const int lane = threadIdx.x & 31;
@@ -56,10 +112,17 @@ __global__ void __launch_bounds__(kEnergyThreads)
     double s = 0.0, c = 0.0;
     unsigned st = 0;
     const int64_t half = (n + 1) / 2;
-    for (int64_t r = w; r < half; r += W) {
-        row_potential(state, mass, n, r, lane, s, c, st);
+    for (int64_t q = w; q < half * S; q += W) {
+        // segment k of the n - 1 pairs of rows r and n - 1 - r
+        const int64_t r = q / S, k = q - r * S;
+        const int64_t a = k * (n - 1) / S, b = (k + 1) * (n - 1) / S, first = n - 1 - r;
         const int64_t r2 = n - 1 - r;
-        if (r2 != r) row_potential(state, mass, n, r2, lane, s, c, st);
+        if (a < first)
+            row_potential(state, mass, n, r, r + 1 + a, r + 1 + (b < first ? b : first), lane, s,
+                          c, st);
+        if (b > first && r2 != r)
+            row_potential(state, mass, n, r2, r2 + 1 + (a > first ? a - first : 0),
+                          r2 + 1 + b - first, lane, s, c, st);
     }
     for (int o = 16; o > 0; o >>= 1) {
         const double s2 = __shfl_xor_sync(0xffffffffu, s, o);
@@ -85,7 +148,7 @@ __global__ void __launch_bounds__(kEnergyThreads)
 
 __global__ void __launch_bounds__(1024)
     energy_final_kernel(const double *state, const double *mass, int64_t n, const double *work,
-                        int64_t W, double *out)
+                        int64_t W, double *out, unsigned *status, unsigned *host_status)
 {
     __shared__ double sh_s[1024], sh_c[1024], sh_t[1024], sh_tc[1024];
     const int t = threadIdx.x;
@@ -120,6 +183,9 @@ __global__ void __launch_bounds__(1024)
         out[0] = es + ec;
         out[1] = sh_t[0] + sh_tc[0];
         out[2] = sh_s[0] + sh_c[0];
+        const unsigned st = *status;
+        *host_status = st;
+        if (st) *status = 0u;
     }
 }
 
@@ -131,13 +197,18 @@ int energy_work_size(int64_t n)
     return 2 * kEnergyBlocks * (kEnergyThreads / 32);
 }
 
-void launch_energy(const double *state, const double *mass, int64_t n, double *work, int nwork,
-                   double *out, unsigned *status, cudaStream_t s)
+void launch_energy(const double *state, const double *mass, int64_t n, double *work, double *out,
+                   unsigned *status, unsigned *host_status, cudaStream_t s)
 {
-    (void)nwork;
-    energy_pairs_kernel<<<kEnergyBlocks, kEnergyThreads, 0, s>>>(state, mass, n, work, status);
-    const int64_t W = (int64_t)kEnergyBlocks * (kEnergyThreads / 32);
-    energy_final_kernel<<<1, 1024, 0, s>>>(state, mass, n, work, W, out);
+    // segments of about 1024 pairs or more, so that the last round of the
+    // warps is short; no more blocks than there are segments for
+    const int S = (int)(n < 2048 ? 1 : (n < 8192 ? n / 1024 : 8));
+    const int64_t items = (n + 1) / 2 * S, per = kEnergyThreads / 32;
+    const int64_t need = (items + per - 1) / per;
+    const int blocks = (int)(need < kEnergyBlocks ? need : kEnergyBlocks);
+    energy_pairs_kernel<<<blocks, kEnergyThreads, 0, s>>>(state, mass, n, S, work, status);
+    energy_final_kernel<<<1, 1024, 0, s>>>(state, mass, n, work, blocks * per, out, status,
+                                           host_status);
 }
 
 }  // namespace sakura

@@ -48,7 +48,8 @@ struct Context {
     cudaStream_t stream = nullptr;
     unsigned *d_status = nullptr;
     unsigned long long *d_stats = nullptr;
-    double *d_energy = nullptr;  // [3] E, T, U
+    double *h_energy = nullptr;      // page-locked [3]: E, T, U
+    double *h_energy_dev = nullptr;  // its address on the device
     unsigned *h_status = nullptr;      // page-locked host copy of the status word
     unsigned *h_status_dev = nullptr;  // its address on the device
     Buffer partial;              // pair-kernel segment sums
@@ -946,7 +947,9 @@ int sakura_init(const sakura_config *cfg)
         if (cudaMalloc(&g.d_stats, sakura::kStatCount * sizeof(unsigned long long)) !=
             cudaSuccess)
             return SAKURA_E_NOMEM;
-        if (cudaMalloc(&g.d_energy, 3 * sizeof(double)) != cudaSuccess) return SAKURA_E_NOMEM;
+        if (cudaHostAlloc(&g.h_energy, 3 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+            cudaHostGetDevicePointer(&g.h_energy_dev, g.h_energy, 0) != cudaSuccess)
+            return SAKURA_E_NOMEM;
         if (cudaMemset(g.d_status, 0, sizeof(unsigned)) != cudaSuccess) return SAKURA_E_CUDA;
         if (cudaHostAlloc(&g.h_status, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
             cudaHostGetDevicePointer(&g.h_status_dev, g.h_status, 0) != cudaSuccess)
@@ -984,7 +987,7 @@ int sakura_finalize(void)
     }
     cudaFree(g.d_status);
     cudaFree(g.d_stats);
-    cudaFree(g.d_energy);
+    if (g.h_energy) cudaFreeHost(g.h_energy);
     if (g.h_status) cudaFreeHost(g.h_status);
     for (auto &p : g.timers) g.spare.push_back(p);
     for (auto &p : g.spare) {
@@ -1090,20 +1093,15 @@ int sakura_energy(const double *state, const double *masses, int64_t n, double *
 {
     if (!g.init) return SAKURA_E_NOINIT;
     if (!state || !masses || n < 1 || !E_out) return SAKURA_E_ARG;
-    const int nwork = sakura::energy_work_size(n);
-    int rc = grow(g.energy_work, (size_t)nwork * sizeof(double));
+    int rc = grow(g.energy_work, (size_t)sakura::energy_work_size(n) * sizeof(double));
     if (rc) return rc;
-    sakura::launch_energy(state, masses, n, (double *)g.energy_work.ptr, nwork, g.d_energy,
-                          g.d_status, g.stream);
+    sakura::launch_energy(state, masses, n, (double *)g.energy_work.ptr, g.h_energy_dev,
+                          g.d_status, g.h_status_dev, g.stream);
     rc = launch_error();
     if (rc) return rc;
-    double out[3];
-    if (cudaMemcpyAsync(out, g.d_energy, sizeof(out), cudaMemcpyDeviceToHost, g.stream) !=
-        cudaSuccess)
-        return SAKURA_E_CUDA;
-    rc = drain_status();
-    *E_out = out[0];
-    return rc;
+    if (cudaStreamSynchronize(g.stream) != cudaSuccess) return SAKURA_E_CUDA;
+    *E_out = *(volatile double *)g.h_energy;
+    return status_to_code(*(volatile unsigned *)g.h_status);
 }
 
 int sakura_step_batched(double *state, const double *masses, const int64_t *offsets,

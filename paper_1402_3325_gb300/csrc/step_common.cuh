@@ -176,8 +176,10 @@ void launch_prep_step(const double *state, const double *mass, double *X, float 
 // W = 0: no pair sums (n = 1)
 void launch_apply_step(double *state, const double *X, const double *partial, int64_t n,
                        int64_t W, double post_drift, unsigned *status, cudaStream_t s);
-void launch_energy(const double *state, const double *mass, int64_t n, double *work,
-                   int nwork, double *out, unsigned *status, cudaStream_t s);
+// out (page-locked host memory): E, T, U; the status word goes to
+// host_status and is cleared
+void launch_energy(const double *state, const double *mass, int64_t n, double *work, double *out,
+                   unsigned *status, unsigned *host_status, cudaStream_t s);
 int energy_work_size(int64_t n);
 
 }  // namespace sakura
