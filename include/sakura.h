@@ -55,7 +55,10 @@ extern "C" {
                                form; pairs outside single-precision range,
                                bound orbits whose step exceeds 0.9 of the
                                period and unconverged pairs are solved in
-                               FP64.  Symmetric pair mode only (else as
+                               FP64.  Pairs that move by less than 2^-5 of
+                               their separation (second-order map) take their
+                               increments' leading term in FP64 and the rest
+                               in double-words.  Symmetric pair mode only (else as
                                FP64); the initial guess is the second-order
                                one (SAKURA_GUESS_LEARNED included).  Results
                                match the FP64 form to about 2^-46 relative
@@ -75,6 +78,10 @@ extern "C" {
                                    the same pair (from a float copy of the drifted
                                    state, second-order start); the FP64 iteration and
                                    its convergence test follow as for every guess.
+                                   In the second-order symmetric step pairs that move by
+                                   less than 2^-5 of their separation are solved as one
+                                   FP64 term and double-word corrections instead, to
+                                   the same accuracy (counted as one evaluation, carried).
                                    Symmetric FP64 step only; elsewhere, and for a pair
                                    whose float solve fails, the second-order guess */
 
@@ -129,7 +136,8 @@ typedef struct sakura_stats {
     int64_t max_iters;    /* largest iteration count of any pair                  */
     int64_t warp_slots;   /* sum over warp batches of 32 x (max lane iterations)  */
     int64_t fp32_pairs;   /* pairs solved on the FP32 pipe: in single precision
-                             (mixed form) or in double-word arithmetic (df64)  */
+                             (mixed form) or in double-word arithmetic (df64;
+                             with an FP64 leading term where that form adds one) */
     int64_t fallbacks;    /* pairs that needed bisection or a restart             */
     int64_t solves;       /* Kepler solves performed (pairs / 2 + diagonal-tile
                              pairs in the symmetric mode)                        */

@@ -338,6 +338,19 @@ bool df64_groups(int64_t n)
     return tile_partial_bytes(n) > kDf64TileMaxBytes;
 }
 
+// Steps whose weakly perturbed pairs take the short solve of
+// kepler_weak.cuh: the FP64 form with the single-precision seed (where the
+// caller leaves the initial value to a float solve; with the other guesses
+// the iteration counts they are asked for stay theirs) and the double-word
+// form, the second-order map it is written for, and a step whose products
+// with ordinary velocities and masses stay in float range.
+bool weak_form(int order, double tau)
+{
+    const bool form = g.cfg.precision == SAKURA_PREC_FP64 ? g.cfg.guess == SAKURA_GUESS_FP32
+                                                          : g.cfg.precision == SAKURA_PREC_DF64;
+    return form && order == 2 && std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18;
+}
+
 // The double-word form in row-group phases (step_df64.cu): prep (drift and
 // three-float copy), pair and apply kernels.
 int step_device_df64_grp(const double *src, double *dst, const double *masses, int64_t n,
@@ -410,18 +423,6 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
     return SAKURA_OK;
 }
 
-// Steps whose weakly perturbed pairs take the short solve of
-// kepler_weak.cuh: the FP64 form with the single-precision seed (where the
-// caller leaves the initial value to a float solve; with the other guesses
-// the iteration counts they are asked for stay theirs), the second-order map
-// it is written for, and a step whose products with ordinary velocities and
-// masses stay in float range.
-bool weak_form(int order, double tau)
-{
-    return g.cfg.precision == SAKURA_PREC_FP64 && g.cfg.guess == SAKURA_GUESS_FP32 &&
-           order == 2 && std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18;
-}
-
 // The FP64 form with each unordered pair once, in row-group phases
 // (step_grp.cu).  prepped: X (and X32) already hold this sub-step's drifted
 // state, written by the previous apply kernel; fuse: the apply kernel also
@@ -431,12 +432,14 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
                          bool mixed = false)
 {
     const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
-    const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
-    const bool seed = g.cfg.guess == SAKURA_GUESS_FP32;
+    const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED &&
+                         g.cfg.precision == SAKURA_PREC_FP64;
+    const bool seed = g.cfg.guess == SAKURA_GUESS_FP32 && g.cfg.precision != SAKURA_PREC_DF64;
     const bool weak = !mixed && weak_form(order, dt);
+    const bool dwf = g.cfg.precision == SAKURA_PREC_DF64;  // weak only
     int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks
                      : (int64_t)g.sm_count *
-                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats)
+                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats, dwf)
                                  : sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed));
     const sakura::GrpLayout L = sakura::make_grp_layout(n, sakura::kFp64GrpShape, blocks);
     // scratch: X[7][n] doubles, row partials [Hmax][6][n], column partials
@@ -491,7 +494,7 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     }
     if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
-        sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, g.stream);
+        sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, dwf, g.stream);
     } else {
         sakura::launch_pair_step_grp(a, L, parts, (int)blocks, stats, g.stream);
     }
@@ -531,17 +534,22 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         if (k == MixedKernel::Fp64Groups)
             return step_device_fp64_grp(src, dst, masses, n, dt, order, false, false, 0.0, true);
     }
-    if (df64 && df64_groups(n)) return step_device_df64_grp(src, dst, masses, n, dt, order);
-    if (!df64 && !mixed && fp64_groups(n))
+    const bool weak = !mixed && weak_form(order, dt);
+    if (df64 && df64_groups(n))
+        return weak ? step_device_fp64_grp(src, dst, masses, n, dt, order, prepped, fuse,
+                                           next_drift)
+                    : step_device_df64_grp(src, dst, masses, n, dt, order);
+    const bool dwf = df64 && weak;  // the double-word form's weak kernel
+    df64 = df64 && !weak;
+    if (!df64 && !dwf && !mixed && fp64_groups(n))
         return step_device_fp64_grp(src, dst, masses, n, dt, order, prepped, fuse, next_drift);
     const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
-    const bool learned = !df64 && !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
-    const bool seed = !df64 && g.cfg.guess == SAKURA_GUESS_FP32;
+    const bool learned = !df64 && !dwf && !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
+    const bool seed = !df64 && !dwf && g.cfg.guess == SAKURA_GUESS_FP32;
     const int64_t nb = (n + 31) / 32;
     const int64_t tiles = nb * (nb + 1) / 2;
-    const bool weak = !df64 && !mixed && weak_form(order, dt);
     const int bps = df64   ? sakura::pair_step_df64_blocks_per_sm(stats)
-                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats)
+                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats, dwf)
                            : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
     // contiguous tile-step ranges for W <= T warps (step_common.cuh)
     const int64_t T = tiles * 32;
@@ -612,7 +620,7 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         sakura::launch_pair_step_df64(a, da, Smax, T, (int)blocks, stats, g.stream);
     } else if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
-        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, g.stream);
+        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, dwf, g.stream);
     } else {
         sakura::launch_pair_step_sym(a, Smax, T, (int)blocks, stats, g.stream);
     }
@@ -665,8 +673,13 @@ bool sym_path(int64_t n)
 }
 
 // Sub-steps whose apply kernel can also drift for the next one: the FP64
-// form on symmetric tiles.
-bool fusable(int64_t n) { return sym_path(n) && g.cfg.precision == SAKURA_PREC_FP64; }
+// form's symmetric kernels, and the double-word form's weak ones.
+bool fusable(int64_t n, int order, double tau)
+{
+    return sym_path(n) &&
+           (g.cfg.precision == SAKURA_PREC_FP64 ||
+            (g.cfg.precision == SAKURA_PREC_DF64 && weak_form(order, tau)));
+}
 
 int step_device(const double *src, double *dst, const double *masses, int64_t n, double dt,
                 int order, bool prepped = false, bool fuse = false, double next_drift = 0.0)
@@ -796,14 +809,14 @@ int run_substeps(const double *src, double *mid, double *dst, const double *mass
     int so;
     const int cnt = substeps(order, w, &so);
     const int64_t total = (int64_t)cnt * nsteps;
-    const bool fuse = fusable(n);
     bool prepped = false;
     for (int64_t k = 0; k < total; ++k) {
         const bool last = k == total - 1;
         const double t = w[k % cnt] * dt;
         const double tn = last ? 0.0 : w[(k + 1) % cnt] * dt;
         const double next_drift = so == 2 ? 0.5 * tn : (so == 1 ? 0.0 : tn);  // as the prep
-        const bool fuse_k = fuse && !last && weak_form(so, t) == weak_form(so, tn);
+        const bool fuse_k =
+            !last && fusable(n, so, t) && weak_form(so, t) == weak_form(so, tn);
         const int rc = step_device(k == 0 ? src : mid, last ? dst : mid,
                                    k == 0 ? masses : step_masses(n), n, t, so, prepped, fuse_k,
                                    next_drift);

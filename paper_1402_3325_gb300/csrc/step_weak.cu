@@ -1,7 +1,7 @@
 // step_weak.cu -- the symmetric FP64 step whose weakly perturbed pairs take
 // the short solve of kepler_weak.cuh (the FP64 form with the
-// single-precision seed, order 2), on the systolic tiles of step_sym.cu and
-// in the row-group layout of step_grp.cu.
+// single-precision seed, and the double-word form; order 2), on the systolic
+// tiles of step_sym.cu and in the row-group layout of step_grp.cu.
 //
 // A warp solves a tile in systolic steps: lane l owns row l and at step k
 // holds the pair with column (l + k) mod 32, the column's sums travelling
@@ -18,7 +18,8 @@
 // out.  ms per step: 16384 bodies (black hole) 20.36 -> 5.18 in row groups,
 // 5.12 on tiles; Plummer 1024 0.109 -> 0.044, 2048 0.358 -> 0.106, 4000
 // 1.30 -> 0.352 (the kernels of step_sym.cu and step_grp.cu with the seed
-// before).
+// before); the double-word form, 16384 bodies with binaries: 8.29 -> 5.37
+// (step_df64.cu before: every pair in 1922 double-word flops).
 #include <cuda_runtime.h>
 
 #include "kepler_df64.cuh"
@@ -38,58 +39,121 @@ constexpr int kWeakInline = 8;
 // entries of a warp's queue on tiles: a segment's, and a rest below one batch
 constexpr int kWeakQueue = 32 * kWeakInline + 31;
 
-// FP64 solve of 32 strong pairs (i, j), one per lane, from the drifted state
-// and its float copy; the twelve products m_j d, -m_i d to out[lane]
-__device__ __noinline__ void weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
-                                               double (*out)[12], unsigned *status, int *iters,
-                                               int *fb, int *carried)
+__device__ __forceinline__ dw split_dw(double x)
+{
+    const float h = __double2float_rn(x);
+    return {h, __double2float_rn(x - (double)h)};
+}
+
+// Solve counts of a lane: evaluations, bisections, Taylor carries,
+// double-word solves.
+struct StrongCount {
+    int iters, fb, carried, dw;
+};
+
+// Solve of 32 strong pairs (i, j), one per lane, from the drifted state; the
+// twelve products m_j d, -m_i d to out[lane].  DW false: the FP64 solver,
+// seeded from the float copy of the state.  DW true (the double-word form):
+// the double-word solver for the pairs it admits, the FP64 solver from the
+// analytic guess for the others.
+template <bool DW>
+__device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
+                                                      double (*out)[12], unsigned *status)
 {
     const int lane = threadIdx.x & 31;
     const int64_t n = a.n;
     const double *X = a.X;
-    const float *X32 = a.X32;
     const KeplerParams kp{a.tol, a.max_iter, a.bisection};
-    PairSolve p;
-    double mi = 0.0, mj = 0.0;
+    StrongCount cnt{0, 0, 0, 0};
+    double rr[3], vv[3], mi = 0.0, mj = 0.0;
     if (valid) {
         mi = X[6 * n + i];
         mj = X[6 * n + j];
-        pair_setup(p, a.tau, mi + mj, X[i] - X[j], X[n + i] - X[n + j],
-                   X[2 * n + i] - X[2 * n + j], X[3 * n + i] - X[3 * n + j],
-                   X[4 * n + i] - X[4 * n + j], X[5 * n + i] - X[5 * n + j], a.pre, -1);
-        float dr[3], dv[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            dr[q] = __fadd_rn(__fsub_rn(X32[q * n + i], X32[q * n + j]),
-                              __fsub_rn(X32[(3 + q) * n + i], X32[(3 + q) * n + j]));
-            dv[q] = __fsub_rn(X32[(6 + q) * n + i], X32[(6 + q) * n + j]);
+            rr[q] = X[q * n + i] - X[q * n + j];
+            vv[q] = X[(3 + q) * n + i] - X[(3 + q) * n + j];
         }
-        const K32 o = k32_phase1(dr, dv, X32[9 * n + i] + X32[9 * n + j], a.ptau32, a.t32, 2);
-        if (o.ok && dbits(p.t) == dbits(a.tau) && !p.done) {
-            p.s = f2d(o.s);
-        } else if (!p.done) {
-            p.s = p.t * p.ir0;
-            const double cq = 0.5 * p.s * (p.eta0 * p.ir0);
-            if (magbits(cq) < 0x3fe0000000000000LL) p.s = fma(-cq, p.s, p.s);
-        }
-    } else {
-        p.done = true;
-        p.beta = p.s = 0.0;
-        p.iters = 0;
-        p.status = 0;
-        p.carried = false;
     }
+    bool need64 = valid;
     double d[6];
-    fp64_solve_warp<true>(p, valid, a.tau, a.post * a.tau, kp, d, *iters, *fb);
+    if (DW) {
+        dw r[3], v[3], m = {0.0f, 0.0f}, dd[6];
+        K32 o;
+        o.ok = false;
+        o.x = o.s = 0.0f;
+        o.iters = 0;
+        if (valid) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                r[q] = split_dw(rr[q]);
+                v[q] = split_dw(vv[q]);
+            }
+            m = split_dw(mi + mj);
+            o = dw_phase1(r, v, m, a.ptau32, a.t32, a.guess);
+        }
+        const bool big = __any_sync(0xffffffffu, o.ok && fabsf(o.x) > 0x1p-8f);
+        int evals = 0;
+        const bool solved = o.ok && dw_phase2(r, v, m, split_dw(a.pre * a.tau), split_dw(a.tau),
+                                              split_dw(a.post * a.tau), o.s, big, dd, evals);
+        if (solved) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) d[q] = (double)dd[q].h + (double)dd[q].l;
+        }
+        need64 = valid && !solved;
+        cnt.iters = o.iters + evals;
+        cnt.dw = solved;
+    }
+    if (!DW || __any_sync(0xffffffffu, need64)) {
+        PairSolve p;
+        if (need64) {
+            pair_setup(p, a.tau, mi + mj, rr[0], rr[1], rr[2], vv[0], vv[1], vv[2], a.pre,
+                       DW ? a.guess : -1);
+            if (!DW) {
+                const float *X32 = a.X32;
+                float dr[3], dv[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    dr[q] = __fadd_rn(__fsub_rn(X32[q * n + i], X32[q * n + j]),
+                                      __fsub_rn(X32[(3 + q) * n + i], X32[(3 + q) * n + j]));
+                    dv[q] = __fsub_rn(X32[(6 + q) * n + i], X32[(6 + q) * n + j]);
+                }
+                const K32 o =
+                    k32_phase1(dr, dv, X32[9 * n + i] + X32[9 * n + j], a.ptau32, a.t32, 2);
+                if (o.ok && dbits(p.t) == dbits(a.tau) && !p.done) {
+                    p.s = f2d(o.s);
+                } else if (!p.done) {
+                    p.s = p.t * p.ir0;
+                    const double cq = 0.5 * p.s * (p.eta0 * p.ir0);
+                    if (magbits(cq) < 0x3fe0000000000000LL) p.s = fma(-cq, p.s, p.s);
+                }
+            }
+        } else {
+            p.done = true;
+            p.beta = p.s = 0.0;
+            p.iters = 0;
+            p.status = 0;
+            p.carried = false;
+        }
+        double d64[6];
+        int iters = 0;
+        fp64_solve_warp<!DW>(p, need64, a.tau, a.post * a.tau, kp, d64, iters, cnt.fb);
+        cnt.iters += iters;
+        if (need64) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) d[q] = d64[q];
+            *status |= p.status;
+            cnt.carried = p.carried;
+        }
+    }
     if (valid) {
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
             out[lane][q] = mj * d[q];
             out[lane][6 + q] = -mi * d[q];
         }
-        *status |= p.status;
     }
-    *carried = valid && p.carried ? 1 : 0;
+    return cnt;
 }
 
 // Per-warp state of the weak pair kernels.
@@ -99,18 +163,19 @@ struct WeakWarp {
     double (*res)[12];        // [32][12] results of a batch of strong solves
     int tail;
     unsigned status;
-    long long it_sum, slots, fallbacks, carries;
+    long long it_sum, slots, fallbacks, carries, ndw;
     int it_max;
 
     template <bool STATS>
-    __device__ __forceinline__ void count(int lane, int iters, int fb, int carried)
+    __device__ __forceinline__ void count(int lane, const StrongCount &c)
     {
         if (STATS) {
-            it_sum += iters;
-            fallbacks += fb;
-            carries += carried;
-            it_max = max(it_max, iters);
-            const int wmax = __reduce_max_sync(0xffffffffu, iters);
+            it_sum += c.iters;
+            fallbacks += c.fb;
+            carries += c.carried;
+            ndw += c.dw;
+            it_max = max(it_max, c.iters);
+            const int wmax = __reduce_max_sync(0xffffffffu, c.iters);
             if (lane == 0) slots += 32LL * wmax;
         }
     }
@@ -126,6 +191,7 @@ struct WeakWarp {
                 slots += __shfl_xor_sync(0xffffffffu, slots, o);
                 fallbacks += __shfl_xor_sync(0xffffffffu, fallbacks, o);
                 carries += __shfl_xor_sync(0xffffffffu, carries, o);
+                ndw += __shfl_xor_sync(0xffffffffu, ndw, o);
                 it_max = max(it_max, __shfl_xor_sync(0xffffffffu, it_max, o));
             }
             if (lane == 0) {
@@ -133,6 +199,7 @@ struct WeakWarp {
                 atomicAdd(&a.stats[kStatSlots], (unsigned long long)slots);
                 atomicAdd(&a.stats[kStatFallbacks], (unsigned long long)fallbacks);
                 atomicAdd(&a.stats[kStatCarries], (unsigned long long)carries);
+                atomicAdd(&a.stats[kStatFp32Pairs], (unsigned long long)ndw);
                 atomicMax(&a.stats[kStatMaxIters], (unsigned long long)it_max);
             }
         }
@@ -143,7 +210,7 @@ struct WeakWarp {
 // and column block 32 J.. (layout indices; L maps them to particles).
 // Returns the tile's sums of the lane's row in row[0..5] and of column
 // (lane + k1 - 1) mod 32 in col[0..5] (positions, then velocities).
-template <bool STATS>
+template <bool STATS, bool DW>
 __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws, int n, bool rev,
                                           int i0, int j0, int k0, int k1, int tag, int lane,
                                           WeakWarp &s, double row[6], double col[6])
@@ -177,7 +244,7 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
         if (STATS) {
             const int any = __any_sync(0xffffffffu, weak);
             s.it_sum += weak ? 1 : 0;
-            s.carries += weak ? 1 : 0;
+            (DW ? s.ndw : s.carries) += weak ? 1 : 0;
             s.it_max = max(s.it_max, weak ? 1 : 0);
             if (lane == 0 && any) s.slots += 32;
         }
@@ -194,10 +261,8 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
                     dirty = true;
                     __syncwarp();
                 }
-                int iters = 0, fb = 0, car = 0;
-                weak_strong_solve(a, strong, rev ? last - i : i, rev ? last - j : j, s.res,
-                                  &s.status, &iters, &fb, &car);
-                s.count<STATS>(lane, iters, fb, car);
+                s.count<STATS>(lane, weak_strong_solve<DW>(a, strong, rev ? last - i : i,
+                                                           rev ? last - j : j, s.res, &s.status));
                 if (strong) {
 #pragma unroll
                     for (int q = 0; q < 6; ++q) {
@@ -244,7 +309,7 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
 // as the queue fills, and what is left at the block's end with the other
 // warps' rests, packed (a warp of a 1024-body step has one or two strong
 // pairs in all).
-template <bool STATS>
+template <bool STATS, bool DW>
 __global__ void __launch_bounds__(128, 3)
     pair_step_weak_kernel(StepArgs a, WeakStep ws, int Smax, int64_t T)
 {
@@ -259,7 +324,7 @@ __global__ void __launch_bounds__(128, 3)
     const int64_t n = a.n;
     const int64_t W = (int64_t)gridDim.x * 4;
     const int64_t w = (int64_t)blockIdx.x * 4 + wib;
-    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0};
+    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0, 0};
 
     // adds the results of entries e0 .. e0 + m - 1 of the queue, at
     // res[r0 ..], to their slots (written before): lane c component c
@@ -287,7 +352,7 @@ __global__ void __launch_bounds__(128, 3)
         int64_t I, J;
         sym_tile_of(tile, I, J);
         double row[6], col[6];
-        weak_tile<STATS>(a, ws, (int)n, false, (int)(32 * I), (int)(32 * J), k0, k1, h, lane, s,
+        weak_tile<STATS, DW>(a, ws, (int)n, false, (int)(32 * I), (int)(32 * J), k0, k1, h, lane, s,
                          row, col);
         // row sums of rows i to slot (J, h); column sums to slot (I, h)
         const int64_t i = 32 * I + lane, j = 32 * J + ((lane + k1 - 1) & 31);
@@ -305,9 +370,8 @@ __global__ void __launch_bounds__(128, 3)
         while (s.tail >= 32) {
             s.tail -= 32;
             const int2 q = s.queue[s.tail + lane];
-            int iters = 0, fb = 0, car = 0;
-            weak_strong_solve(a, true, q.x, q.y & 0xffffff, s.res, &s.status, &iters, &fb, &car);
-            s.count<STATS>(lane, iters, fb, car);
+            s.count<STATS>(lane, weak_strong_solve<DW>(a, true, q.x, q.y & 0xffffff, s.res,
+                                                       &s.status));
             __syncwarp();
             add_results(s.tail, 32, 32 * wib);
             __syncwarp();
@@ -323,9 +387,8 @@ __global__ void __launch_bounds__(128, 3)
         const int o = e < c0 ? 0 : (e < c1 ? 1 : (e < c2 ? 2 : 3));
         const int b0 = o == 0 ? 0 : (o == 1 ? c0 : (o == 2 ? c1 : c2));
         const int2 q = v ? queue[o][e - b0] : make_int2(0, 0);
-        int iters = 0, fb = 0, car = 0;
-        weak_strong_solve(a, v, q.x, q.y & 0xffffff, s.res, &s.status, &iters, &fb, &car);
-        s.count<STATS>(lane, iters, fb, car);
+        s.count<STATS>(lane,
+                       weak_strong_solve<DW>(a, v, q.x, q.y & 0xffffff, s.res, &s.status));
     }
     __syncthreads();
     add_results(0, s.tail, wib == 0 ? 0 : (wib == 1 ? c0 : (wib == 2 ? c1 : c2)));
@@ -352,7 +415,7 @@ constexpr size_t weak_grp_smem()
            sizeof(int2) * kFp64GrpWarps * (32 * kWeakInline * kWeakGrpWindow);
 }
 
-template <bool STATS>
+template <bool STATS, bool DW>
 __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
     pair_step_grp_weak_kernel(StepArgs a, WeakStep ws, GrpLayout L, GrpParts parts)
 {
@@ -377,7 +440,7 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
     const int64_t nb = L.nb;
     const int64_t B = gridDim.x;
     const int64_t b = blockIdx.x;
-    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0};
+    WeakWarp s{queue[wib], sacc[wib], res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0, 0};
 
     GrpPos cur = grp_block_start(L, b, B);
     __shared__ GrpPos s_end;
@@ -408,7 +471,7 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
                 const int64_t I = g * G + r, Jt = J0 + cb;
                 const int kb = cb == 0 ? kfirst : 0;
                 const int ke = cb == wl - 1 ? klast : 32;
-                weak_tile<STATS>(a, ws, (int)n, L.rev != 0, (int)(32 * I), (int)(32 * Jt), kb, ke,
+                weak_tile<STATS, DW>(a, ws, (int)n, L.rev != 0, (int)(32 * I), (int)(32 * Jt), kb, ke,
                                  cb, lane, s, row, col);
                 c = (lane + ke - 1) & 31;
                 if (I == Jt) {
@@ -438,11 +501,10 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
                 int o = 0, eo = e;
                 while (o + 1 < G && eo >= cnt[o]) eo -= cnt[o++];
                 const int2 q = v ? queue[o][eo] : make_int2(0, 0);
-                int iters = 0, fb = 0, car = 0;
-                weak_strong_solve(a, v, (int)grp_particle(L, n, q.x),
-                                  (int)grp_particle(L, n, q.y & 0xffffff), s.res, &s.status,
-                                  &iters, &fb, &car);
-                s.count<STATS>(lane, iters, fb, car);
+                s.count<STATS>(lane, weak_strong_solve<DW>(
+                                         a, v, (int)grp_particle(L, n, q.x),
+                                         (int)grp_particle(L, n, q.y & 0xffffff), s.res,
+                                         &s.status));
             }
             __syncthreads();
             const int m0 = max(base, r0), m1 = min(base + s.tail, r0 + 32 * G);
@@ -508,23 +570,46 @@ __global__ void prep_weak_kernel(const double *state, const double *mass, double
         const double x = fma(v, drift, x0);
         X[q * n + i] = x;
         X[(3 + q) * n + i] = v;
-        const float hi = __double2float_rn(x);
-        X32[q * n + i] = hi;
-        X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
-        X32[(6 + q) * n + i] = __double2float_rn(v);
+        if (X32) {
+            const float hi = __double2float_rn(x);
+            X32[q * n + i] = hi;
+            X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
+            X32[(6 + q) * n + i] = __double2float_rn(v);
+        }
         weak_row_component(rows, n, i, q, x0, v, tau);
     }
     X[6 * n + i] = m;
-    X32[9 * n + i] = __double2float_rn(m);
+    if (X32) X32[9 * n + i] = __double2float_rn(m);
     weak_row_mass(rows, n, i, m, tau);
 }
 
-int pair_step_weak_blocks_per_sm(bool stats)
+namespace {
+
+const void *weak_kernel(bool stats, bool dwf)
 {
-    const void *fn = stats ? (const void *)pair_step_weak_kernel<true>
-                           : (const void *)pair_step_weak_kernel<false>;
+    if (dwf)
+        return stats ? (const void *)pair_step_weak_kernel<true, true>
+                     : (const void *)pair_step_weak_kernel<false, true>;
+    return stats ? (const void *)pair_step_weak_kernel<true, false>
+                 : (const void *)pair_step_weak_kernel<false, false>;
+}
+
+const void *weak_grp_kernel(bool stats, bool dwf)
+{
+    if (dwf)
+        return stats ? (const void *)pair_step_grp_weak_kernel<true, true>
+                     : (const void *)pair_step_grp_weak_kernel<false, true>;
+    return stats ? (const void *)pair_step_grp_weak_kernel<true, false>
+                 : (const void *)pair_step_grp_weak_kernel<false, false>;
+}
+
+}  // namespace
+
+int pair_step_weak_blocks_per_sm(bool stats, bool dwf)
+{
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, 128, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, weak_kernel(stats, dwf), 128, 0) !=
+        cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
@@ -532,20 +617,17 @@ int pair_step_weak_blocks_per_sm(bool stats)
 }
 
 void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
-                           bool stats, cudaStream_t s)
+                           bool stats, bool dwf, cudaStream_t s)
 {
     int Sv = Smax;
     int64_t it = T;
     void *args[] = {(void *)&a, (void *)&ws, (void *)&Sv, (void *)&it};
-    launch_pdl(stats ? (const void *)pair_step_weak_kernel<true>
-                     : (const void *)pair_step_weak_kernel<false>,
-               dim3(blocks), dim3(128), args, 0, s);
+    launch_pdl(weak_kernel(stats, dwf), dim3(blocks), dim3(128), args, 0, s);
 }
 
-int pair_step_grp_weak_blocks_per_sm(bool stats)
+int pair_step_grp_weak_blocks_per_sm(bool stats, bool dwf)
 {
-    const void *fn = stats ? (const void *)pair_step_grp_weak_kernel<true>
-                           : (const void *)pair_step_grp_weak_kernel<false>;
+    const void *fn = weak_grp_kernel(stats, dwf);
     int b = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)weak_grp_smem()) != cudaSuccess ||
@@ -558,10 +640,10 @@ int pair_step_grp_weak_blocks_per_sm(bool stats)
 }
 
 void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
-                               const GrpParts &parts, int blocks, bool stats, cudaStream_t s)
+                               const GrpParts &parts, int blocks, bool stats, bool dwf,
+                               cudaStream_t s)
 {
-    const void *fn = stats ? (const void *)pair_step_grp_weak_kernel<true>
-                           : (const void *)pair_step_grp_weak_kernel<false>;
+    const void *fn = weak_grp_kernel(stats, dwf);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)weak_grp_smem());
     GrpLayout Lv = L;
     GrpParts pv = parts;

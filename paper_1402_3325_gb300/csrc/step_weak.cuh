@@ -14,13 +14,16 @@ struct WeakStep {
     double inv_t;  // 1 / tau
 };
 
+// dwf: the double-word form (its strong pairs take the double-word solver;
+// no float copy X32)
 void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
                       float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s);
 void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
-                           bool stats, cudaStream_t s);
-int pair_step_weak_blocks_per_sm(bool stats);
+                           bool stats, bool dwf, cudaStream_t s);
+int pair_step_weak_blocks_per_sm(bool stats, bool dwf);
 void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
-                               const GrpParts &parts, int blocks, bool stats, cudaStream_t s);
-int pair_step_grp_weak_blocks_per_sm(bool stats);
+                               const GrpParts &parts, int blocks, bool stats, bool dwf,
+                               cudaStream_t s);
+int pair_step_grp_weak_blocks_per_sm(bool stats, bool dwf);
 
 }  // namespace sakura

@@ -1,4 +1,4 @@
-"""The seeded FP64 step's weak pairs (csrc/kepler_weak.cuh, csrc/step_weak.cu)
+"""The weak pairs of the seeded FP64 step and of the double-word form (csrc/kepler_weak.cuh, csrc/step_weak.cu)
 on tiles and in row groups against the oracle, at ragged sizes and for mixes
 of weak and strong pairs."""
 import os
@@ -49,15 +49,16 @@ def _kinds(n):
 
 
 @pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp64", "df64"])
 @pytest.mark.parametrize("n", [21, 32, 33, 64, 95, 129, 1000])
-def test_weak_step_matches_oracle(n, flag):
+def test_weak_step_matches_oracle(n, precision, flag):
     for name, s in _kinds(n):
-        got, st = _step(s, s.dt, flags=flag | 2)
+        got, st = _step(s, s.dt, flags=flag | 2, precision=precision)
         rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
         assert rc == oracle.OK
         _close(got, (r, v))
         assert st["iters"] >= st["solves"]
-        again, _ = _step(s, s.dt, flags=flag | 2)
+        again, _ = _step(s, s.dt, flags=flag | 2, precision=precision)
         assert np.array_equal(got[0], again[0]) and np.array_equal(got[1], again[1])
         if name == "planar":
             assert not got[0][:, 2].any() and not got[1][:, 2].any()
