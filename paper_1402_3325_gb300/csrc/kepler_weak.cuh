@@ -311,6 +311,7 @@ DW_HD float weak_speed2(const WeakParticle &p)
 struct WeakDiff {
     double x[3], r2;
     dw r2d, w[3];
+    float w2, y;  // |w|^2, 1 / r0
 };
 
 // Relative state of the pair and whether it takes weak_add (sa =
@@ -329,12 +330,27 @@ DW_HD bool weak_class(const WeakParticle &a, float sa, const WeakParticle &b, We
         const dw s = two_sum(a.w[q].h, -b.w[q].h);
         d.w[q] = fast_two_sum(s.h, fadd(s.l, fsub(a.w[q].l, b.w[q].l)));
     }
-    const float w2 = ffma(d.w[0].h, d.w[0].h, ffma(d.w[1].h, d.w[1].h, fmul(d.w[2].h, d.w[2].h)));
-    const float y = rsqrt_approx(d.r2d.h), y2 = fmul(y, y);
-    const float mu = fmul(fmul(fadd(a.mh.h, b.mh.h), y), y2);
-    return hi - 0x3c300000u < 0x07800000u && w2 <= fmul(kWeakEps2, d.r2d.h) &&
+    d.w2 = ffma(d.w[0].h, d.w[0].h, ffma(d.w[1].h, d.w[1].h, fmul(d.w[2].h, d.w[2].h)));
+    d.y = rsqrt_approx(d.r2d.h);
+    const float y2 = fmul(d.y, d.y);
+    const float mu = fmul(fmul(fadd(a.mh.h, b.mh.h), d.y), y2);
+    return hi - 0x3c300000u < 0x07800000u && d.w2 <= fmul(kWeakEps2, d.r2d.h) &&
            fadd(sa, weak_speed2(b)) <= fmul(kWeakSpeed2, d.r2d.h) && mu <= kWeakMu &&
            fmul(fminf(a.mh.h, b.mh.h), y2) >= kWeakMin;
+}
+
+// Whether a class test of e < e_max < 1 on float copies (kepler_fp32.cuh) is
+// certain to find the pair unbound, (v^2 - 2 m / r0) h^2 >= 0: v^2 above 2 m
+// / r0 and h^2 = r0^2 v^2 - (r0.v)^2 above 0, each by more than the test's
+// roundings: of v^2 up to 2^-22 |v| (|v_i| + |v_j|), which is at most 2^-10
+// v^2 + 2^-32 (v_i^2 + v_j^2), and of h^2 up to 2^-21 r0^2 v^2.
+DW_HD bool weak_unbound(const WeakParticle &a, float sa, const WeakParticle &b, const WeakDiff &d)
+{
+    const float pot = fmul(fmul(2.0f * 1.004f, fadd(a.mh.h, b.mh.h)), d.y);
+    const float x = dw_split0(d.x[0]).h, y = dw_split0(d.x[1]).h, z = dw_split0(d.x[2]).h;
+    const float xw = ffma(x, d.w[0].h, ffma(y, d.w[1].h, fmul(z, d.w[2].h)));
+    return fmul(d.w2, 0.998f) > ffma(fadd(sa, weak_speed2(b)), 0x1p-30f, pot) &&
+           fmul(xw, xw) < fmul(1.0f - 0x1p-16f, fmul(d.w2, d.r2d.h));
 }
 
 // Adds the pair's increments to the sums of both particles:

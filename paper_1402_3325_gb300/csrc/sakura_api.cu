@@ -343,12 +343,25 @@ bool df64_groups(int64_t n)
 // caller leaves the initial value to a float solve; with the other guesses
 // the iteration counts they are asked for stay theirs) and the double-word
 // form, the second-order map it is written for, and a step whose products
-// with ordinary velocities and masses stay in float range.
+// with ordinary velocities and masses stay in float range.  The mixed form
+// has them under the literal rule with e_max < 1, where only bound pairs are
+// FP32-class: few in a cluster, and told from the others by their energy.
 bool weak_form(int order, double tau)
 {
-    const bool form = g.cfg.precision == SAKURA_PREC_FP64 ? g.cfg.guess == SAKURA_GUESS_FP32
-                                                          : g.cfg.precision == SAKURA_PREC_DF64;
+    const bool seed = g.cfg.guess == SAKURA_GUESS_FP32;
+    const bool form = g.cfg.precision == SAKURA_PREC_FP64   ? seed
+                      : g.cfg.precision == SAKURA_PREC_DF64 ? true
+                                                            : seed &&
+                                          g.cfg.mixed_rule == SAKURA_MIXED_RULE_LITERAL &&
+                                          g.cfg.mixed_e_max < 1.0;
     return form && order == 2 && std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18;
+}
+
+sakura::WeakForm weak_kind()
+{
+    return g.cfg.precision == SAKURA_PREC_DF64    ? sakura::WeakForm::Df64
+           : g.cfg.precision == SAKURA_PREC_MIXED ? sakura::WeakForm::Mixed
+                                                  : sakura::WeakForm::Fp64;
 }
 
 // The double-word form in row-group phases (step_df64.cu): prep (drift and
@@ -435,11 +448,10 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED &&
                          g.cfg.precision == SAKURA_PREC_FP64;
     const bool seed = g.cfg.guess == SAKURA_GUESS_FP32 && g.cfg.precision != SAKURA_PREC_DF64;
-    const bool weak = !mixed && weak_form(order, dt);
-    const bool dwf = g.cfg.precision == SAKURA_PREC_DF64;  // weak only
+    const bool weak = weak_form(order, dt);
     int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks
                      : (int64_t)g.sm_count *
-                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats, dwf)
+                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats, weak_kind())
                                  : sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed));
     const sakura::GrpLayout L = sakura::make_grp_layout(n, sakura::kFp64GrpShape, blocks);
     // scratch: X[7][n] doubles, row partials [Hmax][6][n], column partials
@@ -494,7 +506,8 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     }
     if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
-        sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, dwf, g.stream);
+        sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, weak_kind(),
+                                          g.stream);
     } else {
         sakura::launch_pair_step_grp(a, L, parts, (int)blocks, stats, g.stream);
     }
@@ -534,7 +547,7 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         if (k == MixedKernel::Fp64Groups)
             return step_device_fp64_grp(src, dst, masses, n, dt, order, false, false, 0.0, true);
     }
-    const bool weak = !mixed && weak_form(order, dt);
+    const bool weak = weak_form(order, dt);
     if (df64 && df64_groups(n))
         return weak ? step_device_fp64_grp(src, dst, masses, n, dt, order, prepped, fuse,
                                            next_drift)
@@ -549,7 +562,7 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
     const int64_t nb = (n + 31) / 32;
     const int64_t tiles = nb * (nb + 1) / 2;
     const int bps = df64   ? sakura::pair_step_df64_blocks_per_sm(stats)
-                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats, dwf)
+                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats, weak_kind())
                            : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
     // contiguous tile-step ranges for W <= T warps (step_common.cuh)
     const int64_t T = tiles * 32;
@@ -620,7 +633,8 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         sakura::launch_pair_step_df64(a, da, Smax, T, (int)blocks, stats, g.stream);
     } else if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
-        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, dwf, g.stream);
+        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, weak_kind(),
+                                          g.stream);
     } else {
         sakura::launch_pair_step_sym(a, Smax, T, (int)blocks, stats, g.stream);
     }

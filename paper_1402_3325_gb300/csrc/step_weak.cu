@@ -45,21 +45,28 @@ __device__ __forceinline__ dw split_dw(double x)
     return {h, __double2float_rn(x - (double)h)};
 }
 
-// Solve counts of a lane: evaluations, bisections, Taylor carries,
-// double-word solves.
+// The forms: FP64 with the single-precision seed; double-word; mixed under
+// the literal rule (e_max < 1), seeded.
+constexpr int kWeakFp64 = 0, kWeakDf64 = 1, kWeakMixed = 2;
+
+// Solve counts of a lane: evaluations, bisections, Taylor carries, pairs
+// (double-word form) or ordered pairs (mixed form) solved on the FP32 pipe.
 struct StrongCount {
-    int iters, fb, carried, dw;
+    int iters, fb, carried, n32;
 };
 
 // Solve of 32 strong pairs (i, j), one per lane, from the drifted state; the
-// twelve products m_j d, -m_i d to out[lane].  DW false: the FP64 solver,
-// seeded from the float copy of the state.  DW true (the double-word form):
-// the double-word solver for the pairs it admits, the FP64 solver from the
-// analytic guess for the others.
-template <bool DW>
+// twelve products m_j d, -m_i d to out[lane].  FP64: the FP64 solver, seeded
+// from the float copy of the state.  Double-word: the double-word solver for
+// the pairs it admits, the FP64 solver from the analytic guess for the
+// others.  Mixed: the FP32 solver for the pairs its class rule admits, the
+// seeded FP64 solver for the others.
+template <int MODE>
 __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
-                                                      double (*out)[12], unsigned *status)
+                                                      int weight, double (*out)[12],
+                                                      unsigned *status)
 {
+    constexpr bool DW = MODE == kWeakDf64;
     const int lane = threadIdx.x & 31;
     const int64_t n = a.n;
     const double *X = a.X;
@@ -102,7 +109,30 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
         }
         need64 = valid && !solved;
         cnt.iters = o.iters + evals;
-        cnt.dw = solved;
+        cnt.n32 = solved;
+    }
+    if (MODE == kWeakMixed && valid) {
+        const float *X32 = a.X32;
+        float hi[2][3], lo[2][3], v[2][3], d32[6];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            hi[0][q] = X32[q * n + i];
+            lo[0][q] = X32[(3 + q) * n + i];
+            v[0][q] = X32[(6 + q) * n + i];
+            hi[1][q] = X32[q * n + j];
+            lo[1][q] = X32[(3 + q) * n + j];
+            v[1][q] = X32[(6 + q) * n + j];
+        }
+        Pair32 pr;
+        pair32_setup(pr, hi[0], lo[0], v[0], X32[9 * n + i], hi[1], lo[1], v[1], X32[9 * n + j],
+                     a.rule);
+        int it32 = 0;
+        if (pr.fp32 && pair32_solve(pr, a.t32, a.post32, a.guess, d32, it32)) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) d[q] = (double)d32[q];
+            need64 = false;
+            cnt.n32 = weight;
+        }
     }
     if (!DW || __any_sync(0xffffffffu, need64)) {
         PairSolve p;
@@ -156,6 +186,13 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
     return cnt;
 }
 
+// Ordered pairs that a queue entry stands for: one on a diagonal tile, whose
+// two orders are separate entries, else two.
+__device__ __forceinline__ int strong_weight(int2 q)
+{
+    return (q.x >> 5) == ((q.y & 0xffffff) >> 5) ? 1 : 2;
+}
+
 // Per-warp state of the weak pair kernels.
 struct WeakWarp {
     int2 *queue;              // [kWeakQueue] strong pairs: i, j | tag << 24
@@ -163,7 +200,7 @@ struct WeakWarp {
     double (*res)[12];        // [32][12] results of a batch of strong solves
     int tail;
     unsigned status;
-    long long it_sum, slots, fallbacks, carries, ndw;
+    long long it_sum, slots, fallbacks, carries, n32;
     int it_max;
 
     template <bool STATS>
@@ -173,7 +210,7 @@ struct WeakWarp {
             it_sum += c.iters;
             fallbacks += c.fb;
             carries += c.carried;
-            ndw += c.dw;
+            n32 += c.n32;
             it_max = max(it_max, c.iters);
             const int wmax = __reduce_max_sync(0xffffffffu, c.iters);
             if (lane == 0) slots += 32LL * wmax;
@@ -191,7 +228,7 @@ struct WeakWarp {
                 slots += __shfl_xor_sync(0xffffffffu, slots, o);
                 fallbacks += __shfl_xor_sync(0xffffffffu, fallbacks, o);
                 carries += __shfl_xor_sync(0xffffffffu, carries, o);
-                ndw += __shfl_xor_sync(0xffffffffu, ndw, o);
+                n32 += __shfl_xor_sync(0xffffffffu, n32, o);
                 it_max = max(it_max, __shfl_xor_sync(0xffffffffu, it_max, o));
             }
             if (lane == 0) {
@@ -199,7 +236,7 @@ struct WeakWarp {
                 atomicAdd(&a.stats[kStatSlots], (unsigned long long)slots);
                 atomicAdd(&a.stats[kStatFallbacks], (unsigned long long)fallbacks);
                 atomicAdd(&a.stats[kStatCarries], (unsigned long long)carries);
-                atomicAdd(&a.stats[kStatFp32Pairs], (unsigned long long)ndw);
+                atomicAdd(&a.stats[kStatFp32Pairs], (unsigned long long)n32);
                 atomicMax(&a.stats[kStatMaxIters], (unsigned long long)it_max);
             }
         }
@@ -210,7 +247,7 @@ struct WeakWarp {
 // and column block 32 J.. (layout indices; L maps them to particles).
 // Returns the tile's sums of the lane's row in row[0..5] and of column
 // (lane + k1 - 1) mod 32 in col[0..5] (positions, then velocities).
-template <bool STATS, bool DW>
+template <bool STATS, int MODE>
 __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws, int n, bool rev,
                                           int i0, int j0, int k0, int k1, int tag, int lane,
                                           WeakWarp &s, double row[6], double col[6])
@@ -237,14 +274,18 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
         const WeakParticle B =
             weak_unpack(rows[jl], rows[n + jl], rows[2 * n + jl], rows[3 * n + jl]);
         WeakDiff d;
-        const bool weak = weak_class(A, sa, B, d) && valid;
+        bool weak = weak_class(A, sa, B, d) && valid;
+        // the mixed form's FP32 class holds bound pairs only (e_max < 1):
+        // pairs that are not clearly unbound go to the queue, where the
+        // class rule itself decides
+        if (MODE == kWeakMixed) weak = weak && weak_unbound(A, sa, B, d);
         if (weak) weak_add(A, B, d, vr, er, rr, vc, ec, rc);
         const bool strong = valid && !weak;
         const unsigned mask = __ballot_sync(0xffffffffu, strong);
         if (STATS) {
             const int any = __any_sync(0xffffffffu, weak);
             s.it_sum += weak ? 1 : 0;
-            (DW ? s.ndw : s.carries) += weak ? 1 : 0;
+            (MODE == kWeakDf64 ? s.n32 : s.carries) += weak ? 1 : 0;
             s.it_max = max(s.it_max, weak ? 1 : 0);
             if (lane == 0 && any) s.slots += 32;
         }
@@ -261,8 +302,9 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
                     dirty = true;
                     __syncwarp();
                 }
-                s.count<STATS>(lane, weak_strong_solve<DW>(a, strong, rev ? last - i : i,
-                                                           rev ? last - j : j, s.res, &s.status));
+                s.count<STATS>(lane, weak_strong_solve<MODE>(a, strong, rev ? last - i : i,
+                                                             rev ? last - j : j, diag ? 1 : 2,
+                                                             s.res, &s.status));
                 if (strong) {
 #pragma unroll
                     for (int q = 0; q < 6; ++q) {
@@ -309,7 +351,7 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
 // as the queue fills, and what is left at the block's end with the other
 // warps' rests, packed (a warp of a 1024-body step has one or two strong
 // pairs in all).
-template <bool STATS, bool DW>
+template <bool STATS, int MODE>
 __global__ void __launch_bounds__(128, 3)
     pair_step_weak_kernel(StepArgs a, WeakStep ws, int Smax, int64_t T)
 {
@@ -352,7 +394,7 @@ __global__ void __launch_bounds__(128, 3)
         int64_t I, J;
         sym_tile_of(tile, I, J);
         double row[6], col[6];
-        weak_tile<STATS, DW>(a, ws, (int)n, false, (int)(32 * I), (int)(32 * J), k0, k1, h, lane, s,
+        weak_tile<STATS, MODE>(a, ws, (int)n, false, (int)(32 * I), (int)(32 * J), k0, k1, h, lane, s,
                          row, col);
         // row sums of rows i to slot (J, h); column sums to slot (I, h)
         const int64_t i = 32 * I + lane, j = 32 * J + ((lane + k1 - 1) & 31);
@@ -370,8 +412,8 @@ __global__ void __launch_bounds__(128, 3)
         while (s.tail >= 32) {
             s.tail -= 32;
             const int2 q = s.queue[s.tail + lane];
-            s.count<STATS>(lane, weak_strong_solve<DW>(a, true, q.x, q.y & 0xffffff, s.res,
-                                                       &s.status));
+            s.count<STATS>(lane, weak_strong_solve<MODE>(a, true, q.x, q.y & 0xffffff,
+                                                         strong_weight(q), s.res, &s.status));
             __syncwarp();
             add_results(s.tail, 32, 32 * wib);
             __syncwarp();
@@ -388,7 +430,8 @@ __global__ void __launch_bounds__(128, 3)
         const int b0 = o == 0 ? 0 : (o == 1 ? c0 : (o == 2 ? c1 : c2));
         const int2 q = v ? queue[o][e - b0] : make_int2(0, 0);
         s.count<STATS>(lane,
-                       weak_strong_solve<DW>(a, v, q.x, q.y & 0xffffff, s.res, &s.status));
+                       weak_strong_solve<MODE>(a, v, q.x, q.y & 0xffffff, strong_weight(q), s.res,
+                                               &s.status));
     }
     __syncthreads();
     add_results(0, s.tail, wib == 0 ? 0 : (wib == 1 ? c0 : (wib == 2 ? c1 : c2)));
@@ -415,7 +458,7 @@ constexpr size_t weak_grp_smem()
            sizeof(int2) * kFp64GrpWarps * (32 * kWeakInline * kWeakGrpWindow);
 }
 
-template <bool STATS, bool DW>
+template <bool STATS, int MODE>
 __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
     pair_step_grp_weak_kernel(StepArgs a, WeakStep ws, GrpLayout L, GrpParts parts)
 {
@@ -471,7 +514,7 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
                 const int64_t I = g * G + r, Jt = J0 + cb;
                 const int kb = cb == 0 ? kfirst : 0;
                 const int ke = cb == wl - 1 ? klast : 32;
-                weak_tile<STATS, DW>(a, ws, (int)n, L.rev != 0, (int)(32 * I), (int)(32 * Jt), kb, ke,
+                weak_tile<STATS, MODE>(a, ws, (int)n, L.rev != 0, (int)(32 * I), (int)(32 * Jt), kb, ke,
                                  cb, lane, s, row, col);
                 c = (lane + ke - 1) & 31;
                 if (I == Jt) {
@@ -501,10 +544,10 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
                 int o = 0, eo = e;
                 while (o + 1 < G && eo >= cnt[o]) eo -= cnt[o++];
                 const int2 q = v ? queue[o][eo] : make_int2(0, 0);
-                s.count<STATS>(lane, weak_strong_solve<DW>(
+                s.count<STATS>(lane, weak_strong_solve<MODE>(
                                          a, v, (int)grp_particle(L, n, q.x),
-                                         (int)grp_particle(L, n, q.y & 0xffffff), s.res,
-                                         &s.status));
+                                         (int)grp_particle(L, n, q.y & 0xffffff),
+                                         strong_weight(q), s.res, &s.status));
             }
             __syncthreads();
             const int m0 = max(base, r0), m1 = min(base + s.tail, r0 + 32 * G);
@@ -585,30 +628,31 @@ __global__ void prep_weak_kernel(const double *state, const double *mass, double
 
 namespace {
 
-const void *weak_kernel(bool stats, bool dwf)
+template <int MODE>
+const void *weak_kernel_ptr(bool stats, bool grp)
 {
-    if (dwf)
-        return stats ? (const void *)pair_step_weak_kernel<true, true>
-                     : (const void *)pair_step_weak_kernel<false, true>;
-    return stats ? (const void *)pair_step_weak_kernel<true, false>
-                 : (const void *)pair_step_weak_kernel<false, false>;
+    if (grp)
+        return stats ? (const void *)pair_step_grp_weak_kernel<true, MODE>
+                     : (const void *)pair_step_grp_weak_kernel<false, MODE>;
+    return stats ? (const void *)pair_step_weak_kernel<true, MODE>
+                 : (const void *)pair_step_weak_kernel<false, MODE>;
 }
 
-const void *weak_grp_kernel(bool stats, bool dwf)
+const void *weak_kernel(bool stats, WeakForm form, bool grp)
 {
-    if (dwf)
-        return stats ? (const void *)pair_step_grp_weak_kernel<true, true>
-                     : (const void *)pair_step_grp_weak_kernel<false, true>;
-    return stats ? (const void *)pair_step_grp_weak_kernel<true, false>
-                 : (const void *)pair_step_grp_weak_kernel<false, false>;
+    switch (form) {
+    case WeakForm::Df64: return weak_kernel_ptr<kWeakDf64>(stats, grp);
+    case WeakForm::Mixed: return weak_kernel_ptr<kWeakMixed>(stats, grp);
+    default: return weak_kernel_ptr<kWeakFp64>(stats, grp);
+    }
 }
 
 }  // namespace
 
-int pair_step_weak_blocks_per_sm(bool stats, bool dwf)
+int pair_step_weak_blocks_per_sm(bool stats, WeakForm form)
 {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, weak_kernel(stats, dwf), 128, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, weak_kernel(stats, form, false), 128, 0) !=
         cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -617,17 +661,17 @@ int pair_step_weak_blocks_per_sm(bool stats, bool dwf)
 }
 
 void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
-                           bool stats, bool dwf, cudaStream_t s)
+                           bool stats, WeakForm form, cudaStream_t s)
 {
     int Sv = Smax;
     int64_t it = T;
     void *args[] = {(void *)&a, (void *)&ws, (void *)&Sv, (void *)&it};
-    launch_pdl(weak_kernel(stats, dwf), dim3(blocks), dim3(128), args, 0, s);
+    launch_pdl(weak_kernel(stats, form, false), dim3(blocks), dim3(128), args, 0, s);
 }
 
-int pair_step_grp_weak_blocks_per_sm(bool stats, bool dwf)
+int pair_step_grp_weak_blocks_per_sm(bool stats, WeakForm form)
 {
-    const void *fn = weak_grp_kernel(stats, dwf);
+    const void *fn = weak_kernel(stats, form, true);
     int b = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)weak_grp_smem()) != cudaSuccess ||
@@ -640,10 +684,10 @@ int pair_step_grp_weak_blocks_per_sm(bool stats, bool dwf)
 }
 
 void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
-                               const GrpParts &parts, int blocks, bool stats, bool dwf,
+                               const GrpParts &parts, int blocks, bool stats, WeakForm form,
                                cudaStream_t s)
 {
-    const void *fn = weak_grp_kernel(stats, dwf);
+    const void *fn = weak_kernel(stats, form, true);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)weak_grp_smem());
     GrpLayout Lv = L;
     GrpParts pv = parts;

@@ -14,16 +14,19 @@ struct WeakStep {
     double inv_t;  // 1 / tau
 };
 
-// dwf: the double-word form (its strong pairs take the double-word solver;
-// no float copy X32)
+// The forms that have weak kernels: FP64 with the single-precision seed,
+// double-word (no float copy X32), mixed under the literal rule with e_max < 1
+// and the seed (StepArgs rule, post32).
+enum class WeakForm { Fp64, Df64, Mixed };
+
 void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
                       float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s);
 void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
-                           bool stats, bool dwf, cudaStream_t s);
-int pair_step_weak_blocks_per_sm(bool stats, bool dwf);
+                           bool stats, WeakForm form, cudaStream_t s);
+int pair_step_weak_blocks_per_sm(bool stats, WeakForm form);
 void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &L,
-                               const GrpParts &parts, int blocks, bool stats, bool dwf,
+                               const GrpParts &parts, int blocks, bool stats, WeakForm form,
                                cudaStream_t s);
-int pair_step_grp_weak_blocks_per_sm(bool stats, bool dwf);
+int pair_step_grp_weak_blocks_per_sm(bool stats, WeakForm form);
 
 }  // namespace sakura

@@ -82,3 +82,27 @@ def test_weak_step_orders_and_step_sizes(flag, order, dt):
     got, _ = _step(s, dt, order, 3, flags=flag)
     rc, r, v = oracle.evolve(s.m, s.r, s.v, dt, 3, order, nthreads=NCPU)
     _close(got, (r, v), 1e-10 if dt == 2.0 else 12 * TOL)
+
+
+@pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("kind", ["bh", "radial", "bound"])
+def test_weak_literal_mixed_step_keeps_the_classes(kind, flag):
+    # e_max < 1: bound pairs only; a radially expanding cluster (h^2 = 0 up to
+    # rounding in every pair) and one with every pair bound
+    from paper_1402_3325_gb300 import sakura as sk
+    s = ics.bh_cluster(417, seed=6)
+    if kind == "radial":
+        s.v = 3.0 * s.r
+    if kind == "bound":
+        s = ics.random_cluster(417, seed=6)
+        s.v *= 0.02
+    opts = dict(precision=sk.PREC_MIXED, mixed_rule=sk.MIXED_RULE_LITERAL, flags=flag | 2)
+    got, st = _step(s, s.dt, **opts)
+    import torch
+    classes = sk.pair_classes(torch.tensor(s.soa(), device="cuda"),
+                              torch.tensor(s.m, device="cuda"), s.dt, 2)
+    assert st["fp32_pairs"] == int(classes.sum())
+    rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
+    # a pair in single precision: 2^-21 of its increment, the largest of
+    # which is below 0.02 of the scale here
+    _close(got, (r, v), 1e-8)
