@@ -71,6 +71,13 @@ extern "C" {
 #define SAKURA_PAIRS_SYMMETRIC 1 /* solve every unordered pair once and apply it to
                                     both particles (Newton's third law)            */
 
+/* Initial value of the Kepler iteration.  In the symmetric second-order FP64
+ * step, pairs that move by less than 2^-5 of their separation need none: they
+ * are solved as one FP64 term and double-word corrections, to the same
+ * accuracy.  With SAKURA_GUESS_FP32 they count as one evaluation, carried;
+ * with the other guesses every pair iterates when SAKURA_FLAG_STATS is set
+ * (or kepler_max_iter < 8 or kepler_tol < 1), so that the counts are the
+ * guess's.                                                                  */
 #define SAKURA_GUESS_STANDARD 0 /* s0 = t / r0                               */
 #define SAKURA_GUESS_LEARNED 1  /* s0 from the loaded MLP (sakura_load_mlp)   */
 #define SAKURA_GUESS_TAYLOR 2   /* s0 = (t/r0)(1 - eta0 t / (2 r0^2)): second order in t */
@@ -78,15 +85,13 @@ extern "C" {
                                    the same pair (from a float copy of the drifted
                                    state, second-order start); the FP64 iteration and
                                    its convergence test follow as for every guess.
-                                   In the second-order symmetric step pairs that move by
-                                   less than 2^-5 of their separation are solved as one
-                                   FP64 term and double-word corrections instead, to
-                                   the same accuracy (counted as one evaluation, carried).
                                    Symmetric FP64 step only; elsewhere, and for a pair
                                    whose float solve fails, the second-order guess */
 
 #define SAKURA_FLAG_SYNC_CHECK 1u /* synchronise and report faults on every call */
-#define SAKURA_FLAG_STATS 2u      /* collect iteration statistics (small cost)   */
+#define SAKURA_FLAG_STATS 2u      /* collect iteration statistics (small cost with
+                                     SAKURA_GUESS_FP32; with the other guesses every
+                                     pair then iterates from its guess, see there) */
 #define SAKURA_FLAG_TIMING 4u     /* time every pair-kernel launch with CUDA events */
 #define SAKURA_FLAG_NO_AUTOTUNE 8u /* batched path: skip the block-shape autotuner  */
 #define SAKURA_FLAG_NO_SMALL 16u   /* n <= 20: use the multi-kernel step instead of  */

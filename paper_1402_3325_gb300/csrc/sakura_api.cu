@@ -339,29 +339,35 @@ bool df64_groups(int64_t n)
 }
 
 // Steps whose weakly perturbed pairs take the short solve of
-// kepler_weak.cuh: the FP64 form with the single-precision seed (where the
-// caller leaves the initial value to a float solve; with the other guesses
-// the iteration counts they are asked for stay theirs) and the double-word
-// form, the second-order map it is written for, and a step whose products
-// with ordinary velocities and masses stay in float range.  The mixed form
-// has them under the literal rule with e_max < 1, where only bound pairs are
-// FP32-class: few in a cluster, and told from the others by their energy.
+// kepler_weak.cuh: the second-order map it is written for, a step whose
+// products with ordinary velocities and masses stay in float range, and
+//   - the FP64 form.  With the seed always; with the other guesses unless
+//     statistics are collected, whose iteration counts are to be those of the
+//     guess, and while the Kepler controls are such that the iteration from
+//     any guess would converge on a weak pair (at 2^-5 of the separation it
+//     takes four evaluations to round-off);
+//   - the double-word form;
+//   - the mixed form with the seed under the literal rule with e_max < 1,
+//     where only bound pairs are FP32-class: few in a cluster, and told from
+//     the others by their energy.
 bool weak_form(int order, double tau)
 {
+    if (order != 2 || !(std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18)) return false;
     const bool seed = g.cfg.guess == SAKURA_GUESS_FP32;
-    const bool form = g.cfg.precision == SAKURA_PREC_FP64   ? seed
-                      : g.cfg.precision == SAKURA_PREC_DF64 ? true
-                                                            : seed &&
-                                          g.cfg.mixed_rule == SAKURA_MIXED_RULE_LITERAL &&
-                                          g.cfg.mixed_e_max < 1.0;
-    return form && order == 2 && std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18;
+    if (g.cfg.precision == SAKURA_PREC_DF64) return true;
+    if (g.cfg.precision == SAKURA_PREC_MIXED)
+        return seed && g.cfg.mixed_rule == SAKURA_MIXED_RULE_LITERAL && g.cfg.mixed_e_max < 1.0;
+    return seed || (!(g.cfg.flags & SAKURA_FLAG_STATS) && g.cfg.kepler_max_iter >= 8 &&
+                    g.cfg.kepler_tol >= 1.0);
 }
 
 sakura::WeakForm weak_kind()
 {
-    return g.cfg.precision == SAKURA_PREC_DF64    ? sakura::WeakForm::Df64
-           : g.cfg.precision == SAKURA_PREC_MIXED ? sakura::WeakForm::Mixed
-                                                  : sakura::WeakForm::Fp64;
+    if (g.cfg.precision == SAKURA_PREC_DF64) return sakura::WeakForm::Df64;
+    if (g.cfg.precision == SAKURA_PREC_MIXED) return sakura::WeakForm::Mixed;
+    return g.cfg.guess == SAKURA_GUESS_FP32      ? sakura::WeakForm::Fp64
+           : g.cfg.guess == SAKURA_GUESS_LEARNED ? sakura::WeakForm::Learned
+                                                 : sakura::WeakForm::Guess;
 }
 
 // The double-word form in row-group phases (step_df64.cu): prep (drift and

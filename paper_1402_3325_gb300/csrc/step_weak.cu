@@ -1,7 +1,7 @@
 // step_weak.cu -- the symmetric FP64 step whose weakly perturbed pairs take
-// the short solve of kepler_weak.cuh (the FP64 form with the
-// single-precision seed, and the double-word form; order 2), on the systolic
-// tiles of step_sym.cu and in the row-group layout of step_grp.cu.
+// the short solve of kepler_weak.cuh (the FP64 form, the double-word form and
+// the mixed form under the literal rule; order 2), on the systolic tiles of
+// step_sym.cu and in the row-group layout of step_grp.cu.
 //
 // A warp solves a tile in systolic steps: lane l owns row l and at step k
 // holds the pair with column (l + k) mod 32, the column's sums travelling
@@ -19,7 +19,10 @@
 // 5.12 on tiles; Plummer 1024 0.109 -> 0.044, 2048 0.358 -> 0.106, 4000
 // 1.30 -> 0.352 (the kernels of step_sym.cu and step_grp.cu with the seed
 // before); the double-word form, 16384 bodies with binaries: 8.29 -> 5.37
-// (step_df64.cu before: every pair in 1922 double-word flops).
+// (step_df64.cu before: every pair in 1922 double-word flops); the mixed
+// form's literal rule, 5003 bodies: 2.11 -> 0.56; the default guess, 2999
+// bodies, a fourth-order step on host arrays: 3.26 -> 0.75; the learned
+// guess, 8192 bodies with binaries: 7.07 -> 1.58.
 #include <cuda_runtime.h>
 
 #include "kepler_df64.cuh"
@@ -46,8 +49,9 @@ __device__ __forceinline__ dw split_dw(double x)
 }
 
 // The forms: FP64 with the single-precision seed; double-word; mixed under
-// the literal rule (e_max < 1), seeded.
-constexpr int kWeakFp64 = 0, kWeakDf64 = 1, kWeakMixed = 2;
+// the literal rule (e_max < 1), seeded; FP64 with an analytic guess; FP64
+// with the network's guess.
+constexpr int kWeakFp64 = 0, kWeakDf64 = 1, kWeakMixed = 2, kWeakGuess = 3, kWeakLearned = 4;
 
 // Solve counts of a lane: evaluations, bisections, Taylor carries, pairs
 // (double-word form) or ordered pairs (mixed form) solved on the FP32 pipe.
@@ -60,13 +64,16 @@ struct StrongCount {
 // from the float copy of the state.  Double-word: the double-word solver for
 // the pairs it admits, the FP64 solver from the analytic guess for the
 // others.  Mixed: the FP32 solver for the pairs its class rule admits, the
-// seeded FP64 solver for the others.
+// seeded FP64 solver for the others.  Guess, learned: the FP64 iteration from
+// that guess (the network's weights read from global memory: a batch in a
+// hundred steps or so needs them).
 template <int MODE>
 __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
                                                       int weight, double (*out)[12],
                                                       unsigned *status)
 {
     constexpr bool DW = MODE == kWeakDf64;
+    constexpr bool SEED = MODE == kWeakFp64 || MODE == kWeakMixed;
     const int lane = threadIdx.x & 31;
     const int64_t n = a.n;
     const double *X = a.X;
@@ -138,8 +145,8 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
         PairSolve p;
         if (need64) {
             pair_setup(p, a.tau, mi + mj, rr[0], rr[1], rr[2], vv[0], vv[1], vv[2], a.pre,
-                       DW ? a.guess : -1);
-            if (!DW) {
+                       SEED ? -1 : (MODE == kWeakLearned ? 2 : a.guess));
+            if (SEED) {
                 const float *X32 = a.X32;
                 float dr[3], dv[3];
 #pragma unroll
@@ -165,9 +172,12 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
             p.status = 0;
             p.carried = false;
         }
+        // the batch's result rows serve as the network's staging before them
+        if (MODE == kWeakLearned)
+            learned_guess_warp(p, need64, *a.mlp, reinterpret_cast<__nv_bfloat16 *>(out));
         double d64[6];
         int iters = 0;
-        fp64_solve_warp<!DW>(p, need64, a.tau, a.post * a.tau, kp, d64, iters, cnt.fb);
+        fp64_solve_warp<SEED>(p, need64, a.tau, a.post * a.tau, kp, d64, iters, cnt.fb);
         cnt.iters += iters;
         if (need64) {
 #pragma unroll
@@ -631,11 +641,15 @@ namespace {
 template <int MODE>
 const void *weak_kernel_ptr(bool stats, bool grp)
 {
-    if (grp)
+    if constexpr (MODE == kWeakGuess || MODE == kWeakLearned)  // without statistics only
+        return grp ? (const void *)pair_step_grp_weak_kernel<false, MODE>
+                   : (const void *)pair_step_weak_kernel<false, MODE>;
+    else if (grp)
         return stats ? (const void *)pair_step_grp_weak_kernel<true, MODE>
                      : (const void *)pair_step_grp_weak_kernel<false, MODE>;
-    return stats ? (const void *)pair_step_weak_kernel<true, MODE>
-                 : (const void *)pair_step_weak_kernel<false, MODE>;
+    else
+        return stats ? (const void *)pair_step_weak_kernel<true, MODE>
+                     : (const void *)pair_step_weak_kernel<false, MODE>;
 }
 
 const void *weak_kernel(bool stats, WeakForm form, bool grp)
@@ -643,6 +657,8 @@ const void *weak_kernel(bool stats, WeakForm form, bool grp)
     switch (form) {
     case WeakForm::Df64: return weak_kernel_ptr<kWeakDf64>(stats, grp);
     case WeakForm::Mixed: return weak_kernel_ptr<kWeakMixed>(stats, grp);
+    case WeakForm::Guess: return weak_kernel_ptr<kWeakGuess>(stats, grp);
+    case WeakForm::Learned: return weak_kernel_ptr<kWeakLearned>(stats, grp);
     default: return weak_kernel_ptr<kWeakFp64>(stats, grp);
     }
 }

@@ -16,8 +16,9 @@ struct WeakStep {
 
 // The forms that have weak kernels: FP64 with the single-precision seed,
 // double-word (no float copy X32), mixed under the literal rule with e_max < 1
-// and the seed (StepArgs rule, post32).
-enum class WeakForm { Fp64, Df64, Mixed };
+// and the seed (StepArgs rule, post32), FP64 with an analytic or the learned
+// guess (no X32, no statistics).
+enum class WeakForm { Fp64, Df64, Mixed, Guess, Learned };
 
 void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
                       float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s);

@@ -17,7 +17,11 @@ NCPU = os.cpu_count() or 1
 def _step(s, dt, order=2, nsteps=1, **options):
     import torch
     from paper_1402_3325_gb300 import sakura as sk
-    sk.init(0, stream=torch.cuda.current_stream().cuda_stream, guess=sk.GUESS_FP32, **options)
+    options = {"guess": sk.GUESS_FP32, **options}
+    sk.init(0, stream=torch.cuda.current_stream().cuda_stream, **options)
+    if options["guess"] == sk.GUESS_LEARNED:
+        from paper_1402_3325_gb300 import learned
+        learned.load_default()
     state = torch.tensor(s.soa(), device="cuda")
     mass = torch.tensor(s.m, device="cuda")
     sk.get_stats(reset=True)
@@ -106,3 +110,28 @@ def test_weak_literal_mixed_step_keeps_the_classes(kind, flag):
     # a pair in single precision: 2^-21 of its increment, the largest of
     # which is below 0.02 of the scale here
     _close(got, (r, v), 1e-8)
+
+
+@pytest.mark.parametrize("flag", [32, 64], ids=["tiles", "groups"])
+@pytest.mark.parametrize("guess", [0, 1, 2], ids=["standard", "learned", "taylor"])
+@pytest.mark.parametrize("n", [33, 129, 1000])
+def test_weak_step_with_the_other_guesses(n, guess, flag):
+    # (without statistics: with them every pair iterates from its guess)
+    for name, s in _kinds(n):
+        got, _ = _step(s, s.dt, flags=flag, guess=guess)
+        rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
+        _close(got, (r, v))
+
+
+@pytest.mark.parametrize("guess", [0, 3])
+def test_one_iteration_without_bisection_still_fails_or_carries(guess):
+    # from t / r0 one evaluation converges no pair; the seed's carries
+    from paper_1402_3325_gb300 import sakura as sk
+    s = ics.random_cluster(64, seed=2)
+    if guess == 3:
+        got, _ = _step(s, s.dt, guess=guess, kepler_max_iter=1, kepler_bisection=0)
+        rc, r, v = oracle.step(s.m, s.r, s.v, s.dt, 2, nthreads=NCPU)
+        _close(got, (r, v))
+    else:
+        with pytest.raises(sk.SakuraError):
+            _step(s, s.dt, guess=guess, kepler_max_iter=1, kepler_bisection=0)
