@@ -145,6 +145,28 @@ DW_HD double square_exact(float y)
     return fpb_double((int64_t)((p << (6u - n)) + ((uint64_t)e << 52)));
 }
 
+// a b for normal a, b and a normal product, rounded to nearest (ties up), on
+// the integer pipe: the upper 74 bits of the 106-bit product of the
+// significands (of the lowest partial product only its upper word, an error
+// below 2^-70), normalised and rounded.
+DW_HD double mul_soft(double a, double b)
+{
+    const uint64_t A = (uint64_t)fpb_bits(a), B = (uint64_t)fpb_bits(b);
+    const uint32_t ah = (uint32_t)(A >> 32), al = (uint32_t)A;
+    const uint32_t bh = (uint32_t)(B >> 32), bl = (uint32_t)B;
+    const uint32_t ma = (ah & 0xfffffu) | 0x100000u, mb = (bh & 0xfffffu) | 0x100000u;
+    const uint64_t W = (uint64_t)al * mb + ((uint64_t)ma * bl + (((uint64_t)al * bl) >> 32));
+    const uint64_t H = (uint64_t)ma * mb + (W >> 32);  // in [2^40, 2^42)
+    const uint32_t wl = (uint32_t)W, hl = (uint32_t)H, hh = (uint32_t)(H >> 32);
+    const uint32_t n = hh >> 9, sh = 12u - n;
+    const uint32_t rh = (hh << sh) | (hl >> (32u - sh)), rl = (hl << sh) | (wl >> (32u - sh));
+    const uint32_t up = (wl << sh) >> 31;
+    // the significand's hidden bit adds one to the exponent
+    const uint32_t e = (ah & 0x7ff00000u) + (bh & 0x7ff00000u) + (n << 20) - (1024u << 20);
+    const uint64_t r = (((uint64_t)(rh + e) << 32) | rl) + up;
+    return fpb_double((int64_t)(r | ((uint64_t)((ah ^ bh) & 0x80000000u) << 32)));
+}
+
 // h + l as a double; an exact zero stays zero
 DW_HD double dw_to_double(dw x)
 {
@@ -238,15 +260,13 @@ DW_HD void weak_solve(double r2, dw r2d, const dw xd[3], const dw w[3], dw M, We
     dw F = two_sum(um, fmul(0.5f, a.h));
     F.l = ffma(0.5f, a.l, F.l);
     F = dwu_add(F, dwu_add(ah2, T2));
-    F = two_sum(F.h, F.l);
     dw pr = two_sum(a.h, fmul(0.5f, z.h));
     pr.l = fadd(pr.l, ffma(0.5f, z.l, a.l));
     pr = dwu_norm(dwu_add(pr, dwu_add(ag1, zh2)));
     // delta = F / (1 + p)
     float ir = rcp_approx(fadd(1.0f, pr.h));
-    const float Fh = F.h;
-    const float d1 = fmul(Fh, ir);
-    const float rem = fadd(ffma(-d1, pr.h, fsub(Fh, d1)), F.l);
+    const float d1 = fmul(fadd(F.h, F.l), ir);
+    const float rem = fadd(ffma(-d1, pr.h, fsub(F.h, d1)), F.l);
     const float d2 = fmul(rem, ir);
     // carry to the root
     const float xc2 = fmul(Xf, fadd(0.5f, k2.h));
@@ -364,7 +384,10 @@ DW_HD void weak_add(const WeakParticle &a, const WeakParticle &b, const WeakDiff
     const dw xd[3] = {dw_split0(d.x[0]), dw_split0(d.x[1]), dw_split0(d.x[2])};
     WeakPair o;
     weak_solve(d.r2, d.r2d, xd, d.w, dwu_add(a.mh, b.mh), o);
-    const double qj = b.mt * o.Q, qi = a.mt * o.Q;
+    // on the integer pipe (about 20 instructions): 3 % of a step on tiles at
+    // 4000 bodies, 1 % in row groups at 16384.  The other two multiplies (y^3,
+    // z^2) there too gained nothing more.
+    const double qj = mul_soft(b.mt, o.Q), qi = mul_soft(a.mt, o.Q);
     for (int q = 0; q < 3; ++q) {
         vr[q] = fma(-qj, d.x[q], vr[q]);
         vc[q] = fma(-qi, d.x[q], vc[q]);

@@ -145,3 +145,16 @@ def test_exact_coordinates_and_squares(lib):
     z = np.array([1e-40, -1e-300, 5e-324])
     lib.weak_splits(ctypes.c_long(3), _p(z), _p(out))
     assert np.all(out[:3] == 0)
+
+
+def test_integer_product_is_the_rounded_one(lib):
+    rng = np.random.default_rng(2)
+    a = rng.choice([-1.0, 1.0], 40000) * rng.uniform(1, 2, 40000) * 2.0 ** rng.integers(-300, 300, 40000)
+    b = rng.choice([-1.0, 1.0], 40000) * rng.uniform(1, 2, 40000) * 2.0 ** rng.integers(-300, 300, 40000)
+    edge = np.array([1.0, 1.0 + 2.0 ** -52, 1.5, 2.0 - 2.0 ** -52, 1.0 + 2.0 ** -26])
+    a[:25], b[:25] = np.repeat(edge, 5), np.tile(edge, 5)
+    out = np.zeros(40000)
+    lib.weak_products(ctypes.c_long(40000), _p(a), _p(b), _p(out))
+    # equal but for exact ties, which go up here and to even there
+    off = out != a * b
+    assert off.sum() <= 25 and np.all(np.abs(out - a * b) <= 2.0 ** -52 * np.abs(a * b))

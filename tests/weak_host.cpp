@@ -64,3 +64,8 @@ extern "C" void weak_splits(long n, const double *x, double *out)
         out[k] = (double)s.h + (double)s.l;
     }
 }
+
+extern "C" void weak_products(long n, const double *a, const double *b, double *out)
+{
+    for (long k = 0; k < n; ++k) out[k] = mul_soft(a[k], b[k]);
+}
