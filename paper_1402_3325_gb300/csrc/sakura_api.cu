@@ -692,6 +692,96 @@ bool sym_path(int64_t n)
                            : tile_partial_bytes(n)) <= kSymMaxBytes;
 }
 
+// Tile-steps per warp of the small weak kernel: 2, 4 or 8, the fewest that
+// keep the grid at one, two or three blocks per SM; 0 where it is not used.
+// More of them lengthen a warp's chain (0.5 us each), fewer make more blocks
+// and partial sums than the SMs take at once.  Four steps of a run in us with
+// (2; 4; 8 per warp; the general tile kernel) on 152 SMs: 256 bodies (49; 51;
+// 66; 83), 320 (56; 54; 68; 136), 512 (120; 90; 90; 135), 576 (-; 107; 110;
+// 135), 760 (-; 146; 113; 155), 928 (-; -; 151; 167); 1024 (-; -; 190; 175).
+int weak_small_steps(int64_t n, int order, double tau)
+{
+    if (g.cfg.grid_blocks > 0 || !sym_path(n) || !weak_form(order, tau)) return 0;
+    if (g.cfg.precision == SAKURA_PREC_MIXED ? mixed_kernel(n) != MixedKernel::Tiles
+        : g.cfg.precision == SAKURA_PREC_DF64 ? df64_groups(n)
+                                              : fp64_groups(n))
+        return 0;
+    const int64_t nb = (n + 31) / 32, tiles = nb * (nb + 1) / 2;
+    for (int k = 1; k <= 3; ++k)
+        if ((tiles * 8 >> k) <= k * (int64_t)g.sm_count) return 1 << k;
+    return 0;
+}
+
+// The same for a run whose sub-steps have these time weights.
+int weak_small_run(int64_t n, int order, double dt, const double *w, int cnt)
+{
+    int steps = 0;
+    for (int k = 0; k < cnt; ++k)
+        if (!(steps = weak_small_steps(n, order, w[k] * dt))) return 0;
+    return steps;
+}
+
+// A weak step of a small system (step_weak.cu): pair and apply kernels.
+int step_weak_small(const double *src, double *dst, const double *masses, int64_t n, double dt,
+                    int steps)
+{
+    const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
+    const int64_t nb = (n + 31) / 32, tiles = nb * (nb + 1) / 2, slots = nb * (8 / steps);
+    // scratch: X[7][n] (its last row the copy of host masses), partials
+    // [slots][6][n]
+    int rc = grow(g.partial, (size_t)(7 * n + slots * 6 * n) * sizeof(double));
+    if (rc) return rc;
+    sakura::StepArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.partial = (double *)g.partial.ptr + 7 * n;
+    a.n = n;
+    a.tau = dt;
+    a.pre = a.post = 0.5;
+    a.ptau32 = (float)(a.pre * dt);
+    a.t32 = (float)dt;
+    a.tol = g.cfg.kepler_tol * DBL_EPSILON;
+    a.max_iter = g.cfg.kepler_max_iter;
+    a.bisection = g.cfg.kepler_bisection;
+    a.guess = (g.cfg.guess == SAKURA_GUESS_TAYLOR || g.cfg.guess == SAKURA_GUESS_FP32) ? 2 : 0;
+    a.mlp = g.cfg.precision == SAKURA_PREC_FP64 && g.cfg.guess == SAKURA_GUESS_LEARNED
+                ? (const sakura::MlpWeights *)g.mlp.ptr
+                : nullptr;
+    a.status = g.d_status;
+    a.stats = g.d_stats;
+    if (g.cfg.precision == SAKURA_PREC_MIXED) {
+        a.mixed = 2;
+        a.rule = class_rule(a.pre * dt);
+        a.post32 = (float)a.post;
+    }
+    const sakura::WeakSmall ws{src, masses, 1.0 / dt, steps};
+    const bool timing = (g.cfg.flags & SAKURA_FLAG_TIMING) != 0;
+    std::pair<cudaEvent_t, cudaEvent_t> tm{nullptr, nullptr};
+    if (timing) {
+        tm = take_timer();
+        cudaEventRecord(tm.first, g.stream);
+    }
+    const int64_t blocks = tiles * (8 / steps);
+    sakura::launch_pair_step_weak_small(a, ws, (int)blocks, blocks > 2 * (int64_t)g.sm_count,
+                                        stats, weak_kind(), g.stream);
+    if (timing) {
+        cudaEventRecord(tm.second, g.stream);
+        g.timers.push_back(tm);
+    }
+    sakura::launch_apply_weak_small(src, dst, a.partial, (int)n, (int)slots, dt, g.d_status,
+                                    g.stream);
+    rc = launch_error();
+    if (rc) return rc;
+    g.steps += 1;
+    g.pairs += n * (n - 1);
+    int64_t diag = 0;  // ordered pairs inside diagonal tiles
+    for (int64_t b = 0; b < nb; ++b) {
+        const int64_t nbk = std::min<int64_t>(32, n - 32 * b);
+        diag += nbk * (nbk - 1);
+    }
+    g.solves += (n * (n - 1) - diag) / 2 + diag;
+    return SAKURA_OK;
+}
+
 // Sub-steps whose apply kernel can also drift for the next one: the FP64
 // form's symmetric kernels, and the double-word form's weak ones.
 bool fusable(int64_t n, int order, double tau)
@@ -829,6 +919,24 @@ int run_substeps(const double *src, double *mid, double *dst, const double *mass
     int so;
     const int cnt = substeps(order, w, &so);
     const int64_t total = (int64_t)cnt * nsteps;
+    const int steps = weak_small_run(n, so, dt, w, cnt);
+    if (steps > 0) {
+        if (src != mid) {  // host memory
+            const int rc = grow(g.partial, (size_t)(7 * n + (n + 31) / 32 * (8 / steps) * 6 * n) *
+                                               sizeof(double));
+            if (rc) return rc;
+            sakura::launch_copy_state(src, masses, mid, (double *)step_masses(n), (int)n,
+                                      g.stream);
+            src = mid;
+            masses = step_masses(n);
+        }
+        for (int64_t k = 0; k < total; ++k) {
+            const int rc = step_weak_small(k == 0 ? src : mid, k == total - 1 ? dst : mid, masses,
+                                           n, w[k % cnt] * dt, steps);
+            if (rc) return rc;
+        }
+        return SAKURA_OK;
+    }
     bool prepped = false;
     for (int64_t k = 0; k < total; ++k) {
         const bool last = k == total - 1;
@@ -1090,11 +1198,13 @@ int sakura_evolve_host(double *state, const double *masses, int64_t n, double dt
         return drain_status();
     }
     if (hs && hm) {
-        // sub-steps between the first and the last run in library memory
+        // sub-steps between the first and the last run in library memory, as
+        // do small systems, whose blocks all read the state
         double w[sakura::kMaxSubsteps];
         int so;
         double *ds = nullptr;
-        if ((int64_t)substeps(order, w, &so) * nsteps > 1) {
+        const int cnt = substeps(order, w, &so);
+        if ((int64_t)cnt * nsteps > 1 || weak_small_run(n, so, dt, w, cnt) > 0) {
             rc = grow(g.host_state, sbytes);
             if (rc) return rc;
             ds = (double *)g.host_state.ptr;

@@ -636,6 +636,208 @@ __global__ void prep_weak_kernel(const double *state, const double *mass, double
     weak_row_mass(rows, n, i, m, tau);
 }
 
+// Small systems (up to 928 bodies on 152 SMs): a step is two kernels of a few
+// microseconds each, bound by the latencies of launches, loads and solves and
+// not by any rate, so the chain between them is kept short.  A block takes
+// 4 K consecutive tile-steps of one tile, K = 2, 4 or 8 per warp.  It
+// prepares the tile's 64 particles from the state
+// itself, in shared memory (no drift kernel; the solves then read shared
+// memory), and adds its warps' sums there, so that it leaves one partial sum
+// per tile and block: S = 32 / (4 K) slots per tile, slot (J, h) with the row
+// sums of the rows' particles, slot (I, h) with the column sums of the
+// columns'.  Within the block layout indices are local: rows 0 .. 31, columns
+// 32 .. 63 (a diagonal tile: 0 .. 31).  PER_SM 2: up to 255 registers, no
+// spills; 3 where the grid needs three blocks per SM to be resident at once.
+// Four steps of a run and a copy of the state before them in us, pair kernel
+// on general tiles with drift, pair and apply kernels before -> now: 128
+// bodies 70 -> 43, 512 135 -> 90, 760 155 -> 114, 928 181 -> 151; where most
+// pairs are strong, 128 bodies 95 -> 67 (seeded FP64; the other forms alike).
+struct WeakSmallShared {
+    float4 rows[4 * 64];
+    double X[7 * 64];
+    float X32[10 * 64];
+    double sacc[4][12][32];
+    double res[128][12];
+    int2 queue[4][kWeakQueue];
+    int cnt[4];
+    StepArgs args;
+};
+
+template <bool STATS, int MODE, int PER_SM>
+__global__ void __launch_bounds__(128, PER_SM)
+    pair_step_weak_small_kernel(const __grid_constant__ StepArgs a, WeakSmall ws)
+{
+    __shared__ WeakSmallShared sh;
+    constexpr bool F32 = MODE == kWeakFp64 || MODE == kWeakMixed;
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const int tid = threadIdx.x;
+    const int n = (int)a.n;
+    const int per = 4 * ws.steps, S = 32 / per;
+    const int tile = blockIdx.x / S, h = blockIdx.x - S * tile;
+    int64_t I, J;
+    sym_tile_of(tile, I, J);
+    const int i0 = 32 * (int)I, j0 = 32 * (int)J;
+    const bool diag = I == J;
+    const int nl = diag ? min(32, n - i0) : 32 + min(32, n - j0);
+    griddep_wait();
+    griddep_launch();
+    for (int e = tid; e < 4 * 64; e += 128) {
+        const int q = e >> 6, t = e & 63;
+        if (t >= nl) continue;
+        const int i = t < 32 ? i0 + t : j0 + t - 32;
+        if (q == 3) {
+            const double m = ws.mass[i];
+            if (!(m > 0.0)) atomicOr(a.status, kStatusMass);
+            sh.X[6 * nl + t] = m;
+            if (F32) sh.X32[9 * nl + t] = __double2float_rn(m);
+            weak_row_mass(sh.rows, nl, t, m, a.tau);
+            continue;
+        }
+        const double x0 = ws.src[q * n + i], v = ws.src[(3 + q) * n + i];
+        const double x = fma(v, 0.5 * a.tau, x0);
+        sh.X[q * nl + t] = x;
+        sh.X[(3 + q) * nl + t] = v;
+        if (F32) {
+            const float hi = __double2float_rn(x);
+            sh.X32[q * nl + t] = hi;
+            sh.X32[(3 + q) * nl + t] = __double2float_rn(x - (double)hi);
+            sh.X32[(6 + q) * nl + t] = __double2float_rn(v);
+        }
+        weak_row_component(sh.rows, nl, t, q, x0, v, a.tau);
+    }
+    if (tid == 0) {
+        sh.args = a;
+        sh.args.X = sh.X;
+        sh.args.X32 = F32 ? sh.X32 : nullptr;
+        sh.args.n = nl;
+    }
+    __syncthreads();
+
+    const StepArgs &b = sh.args;
+    const WeakStep wl{sh.rows, ws.inv_t};
+    double(*sacc)[32] = sh.sacc[wib];
+    WeakWarp s{sh.queue[wib], sacc, sh.res + 32 * wib, 0, 0u, 0, 0, 0, 0, 0, 0};
+    auto add_results = [&](int e0, int m, int r0) {
+        for (int e = 0; e < m; ++e) {
+            const int2 q = s.queue[e0 + e];
+            const int i = q.x, j = q.y & 0xffffff;
+            if (lane < (diag ? 6 : 12)) sacc[lane][(lane < 6 ? i : j) & 31] += sh.res[r0 + e][lane];
+        }
+    };
+    {
+        const int k0 = h * per + wib * ws.steps, k1 = k0 + ws.steps;
+        double row[6], col[6];
+        weak_tile<STATS, MODE>(b, wl, nl, false, 0, diag ? 0 : 32, k0, k1, 0, lane, s, row, col);
+        const int c = (lane + k1 - 1) & 31;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            sacc[q][lane] = row[q];
+            sacc[6 + q][c] = col[q];
+        }
+    }
+    __syncwarp();
+    while (s.tail >= 32) {
+        s.tail -= 32;
+        const int2 q = s.queue[s.tail + lane];
+        s.count<STATS>(lane, weak_strong_solve<MODE>(b, true, q.x, q.y & 0xffffff,
+                                                     strong_weight(q), s.res, &s.status));
+        __syncwarp();
+        add_results(s.tail, 32, 32 * wib);
+        __syncwarp();
+    }
+    // the rests of the block's four queues, packed into batches
+    if (lane == 0) sh.cnt[wib] = s.tail;
+    __syncthreads();
+    const int c0 = sh.cnt[0], c1 = c0 + sh.cnt[1], c2 = c1 + sh.cnt[2], tot = c2 + sh.cnt[3];
+    if (tot) {
+        if (32 * wib < tot) {
+            const int e = 32 * wib + lane;
+            const bool v = e < tot;
+            const int o = e < c0 ? 0 : (e < c1 ? 1 : (e < c2 ? 2 : 3));
+            const int b0 = o == 0 ? 0 : (o == 1 ? c0 : (o == 2 ? c1 : c2));
+            const int2 q = v ? sh.queue[o][e - b0] : make_int2(0, 0);
+            s.count<STATS>(lane,
+                           weak_strong_solve<MODE>(b, v, q.x, q.y & 0xffffff, strong_weight(q),
+                                                   s.res, &s.status));
+        }
+        __syncthreads();
+        add_results(0, s.tail, wib == 0 ? 0 : (wib == 1 ? c0 : (wib == 2 ? c1 : c2)));
+        __syncthreads();
+    }
+    for (int e = tid; e < (diag ? 6 : 12) * 32; e += 128) {
+        const int q = e >> 5, l = e & 31;
+        const int i = (q < 6 ? i0 : j0) + l;
+        const double sum = (sh.sacc[0][q][l] + sh.sacc[1][q][l]) +
+                           (sh.sacc[2][q][l] + sh.sacc[3][q][l]);
+        const int64_t slot = (q < 6 ? J : I) * S + h;
+        if (i < n) a.partial[(slot * 6 + (q < 6 ? q : q - 6)) * n + i] = sum;
+    }
+    s.finish<STATS>(a, lane);
+}
+
+// Eqs. 27b-d after pair_step_weak_small_kernel: block (P, q) takes 32
+// particles and the components q, 3 + q; its warps sum the slots w, w + 8,
+// ... of the slots = nb S, four loads in flight, and warp 0 adds the warps'
+// sums in order.  The drift is that of the pair kernel's blocks, from the
+// state again.  src may be dst.
+constexpr int kSmallApplyWarps = 8;
+
+__global__ void __launch_bounds__(32 * kSmallApplyWarps)
+    apply_weak_small_kernel(const double *src, double *dst, const double *partial, int n,
+                            int slots, double tau, unsigned *status)
+{
+    __shared__ double red[kSmallApplyWarps][2][32];
+    griddep_wait();
+    griddep_launch();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int q = blockIdx.y;
+    const int i = 32 * blockIdx.x + lane;
+    double x0 = 0.0, v = 0.0;
+    if (wid == 0 && i < n) {
+        x0 = src[q * n + i];
+        v = src[(3 + q) * n + i];
+    }
+    double er = 0.0, ev = 0.0;
+    if (i < n) {
+        const double *p = partial + q * n + i;
+#pragma unroll 4
+        for (int k = wid; k < slots; k += kSmallApplyWarps) {
+            er += p[(int64_t)k * 6 * n];
+            ev += p[((int64_t)k * 6 + 3) * n];
+        }
+    }
+    red[wid][0][lane] = er;
+    red[wid][1][lane] = ev;
+    __syncthreads();
+    if (wid != 0 || i >= n) return;
+    double r[4], w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        r[k] = red[2 * k][0][lane] + red[2 * k + 1][0][lane];
+        w[k] = red[2 * k][1][lane] + red[2 * k + 1][1][lane];
+    }
+    const double v1 = v + ((w[0] + w[1]) + (w[2] + w[3]));
+    const double x = fma(v, 0.5 * tau, x0) + ((r[0] + r[1]) + (r[2] + r[3]));
+    const double x1 = fma(v1, 0.5 * tau, x);
+    if (!isfinite(x1) || !isfinite(v1)) atomicOr(status, kStatusNonfinite);
+    dst[q * n + i] = x1;
+    dst[(3 + q) * n + i] = v1;
+}
+
+// The state and the masses of host memory, for the blocks of the small
+// kernel that each read them again.
+__global__ void copy_state_kernel(const double *src, const double *mass, double *dst, double *mdst,
+                                  int n)
+{
+    griddep_launch();
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < 6 * n)
+        dst[e] = src[e];
+    else if (e < 7 * n)
+        mdst[e - 6 * n] = mass[e - 6 * n];
+}
+
 namespace {
 
 template <int MODE>
@@ -663,7 +865,52 @@ const void *weak_kernel(bool stats, WeakForm form, bool grp)
     }
 }
 
+template <int MODE, int PER_SM>
+const void *weak_small_ptr(bool stats)
+{
+    if constexpr (MODE == kWeakGuess || MODE == kWeakLearned)
+        return (const void *)pair_step_weak_small_kernel<false, MODE, PER_SM>;
+    else
+        return stats ? (const void *)pair_step_weak_small_kernel<true, MODE, PER_SM>
+                     : (const void *)pair_step_weak_small_kernel<false, MODE, PER_SM>;
+}
+
+template <int PER_SM>
+const void *weak_small_kernel(bool stats, WeakForm form)
+{
+    switch (form) {
+    case WeakForm::Df64: return weak_small_ptr<kWeakDf64, PER_SM>(stats);
+    case WeakForm::Mixed: return weak_small_ptr<kWeakMixed, PER_SM>(stats);
+    case WeakForm::Guess: return weak_small_ptr<kWeakGuess, PER_SM>(stats);
+    case WeakForm::Learned: return weak_small_ptr<kWeakLearned, PER_SM>(stats);
+    default: return weak_small_ptr<kWeakFp64, PER_SM>(stats);
+    }
+}
+
 }  // namespace
+
+void launch_pair_step_weak_small(const StepArgs &a, const WeakSmall &ws, int blocks, bool three,
+                                 bool stats, WeakForm form, cudaStream_t s)
+{
+    void *args[] = {(void *)&a, (void *)&ws};
+    launch_pdl(three ? weak_small_kernel<3>(stats, form) : weak_small_kernel<2>(stats, form),
+               dim3(blocks), dim3(128), args, 0, s);
+}
+
+void launch_apply_weak_small(const double *src, double *dst, const double *partial, int n,
+                             int slots, double tau, unsigned *status, cudaStream_t s)
+{
+    void *args[] = {(void *)&src, (void *)&dst, (void *)&partial, (void *)&n,
+                    (void *)&slots, (void *)&tau, (void *)&status};
+    launch_pdl((const void *)apply_weak_small_kernel, dim3((unsigned)((n + 31) / 32), 3),
+               dim3(32 * kSmallApplyWarps), args, 0, s);
+}
+
+void launch_copy_state(const double *src, const double *mass, double *dst, double *mdst, int n,
+                       cudaStream_t s)
+{
+    copy_state_kernel<<<(7 * n + 127) / 128, 128, 0, s>>>(src, mass, dst, mdst, n);
+}
 
 int pair_step_weak_blocks_per_sm(bool stats, WeakForm form)
 {

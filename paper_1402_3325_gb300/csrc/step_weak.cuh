@@ -30,4 +30,21 @@ void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpL
                                cudaStream_t s);
 int pair_step_grp_weak_blocks_per_sm(bool stats, WeakForm form);
 
+// The small kernel: the state and the masses before the step, and the
+// tile-steps of a warp (2, 4 or 8; a block takes four times as many, the grid
+// 32 / (4 steps) blocks per tile).
+struct WeakSmall {
+    const double *src, *mass;
+    double inv_t;  // 1 / tau
+    int steps;
+};
+
+// three: room for three blocks per SM instead of two
+void launch_pair_step_weak_small(const StepArgs &a, const WeakSmall &ws, int blocks, bool three,
+                                 bool stats, WeakForm form, cudaStream_t s);
+void launch_apply_weak_small(const double *src, double *dst, const double *partial, int n,
+                             int slots, double tau, unsigned *status, cudaStream_t s);
+void launch_copy_state(const double *src, const double *mass, double *dst, double *mdst, int n,
+                       cudaStream_t s);
+
 }  // namespace sakura

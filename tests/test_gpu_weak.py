@@ -135,3 +135,30 @@ def test_one_iteration_without_bisection_still_fails_or_carries(guess):
     else:
         with pytest.raises(sk.SakuraError):
             _step(s, s.dt, guess=guess, kepler_max_iter=1, kepler_bisection=0)
+
+
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp64", "df64"])
+@pytest.mark.parametrize("n", [21, 256, 257, 512, 513, 736, 768, 769, 928, 929])
+def test_small_weak_step_at_the_ends_of_its_ranges(n, precision):
+    # 2, 4 and 8 tile-steps per warp (152 SMs), then the general tile kernel,
+    # which grid_blocks forces too
+    s = ics.random_cluster(n, seed=n, mass_spread=3.0)
+    got, _ = _step(s, s.dt, 4, 2, precision=precision)
+    general, _ = _step(s, s.dt, 4, 2, precision=precision, grid_blocks=7)
+    rc, r, v = oracle.evolve(s.m, s.r, s.v, s.dt, 2, 4, nthreads=NCPU)
+    assert rc == oracle.OK
+    _close(got, (r, v), 12 * TOL)
+    _close(got, general, 12 * TOL)
+
+
+@pytest.mark.parametrize("order,nsteps", [(2, 1), (2, 2), (4, 1)])
+def test_small_weak_step_on_pinned_host_arrays(order, nsteps):
+    import torch
+    from paper_1402_3325_gb300 import sakura as sk
+    s = ics.plummer(100, seed=3)
+    ref, _ = _step(s, s.dt, order, nsteps)
+    state = torch.tensor(s.soa()).pin_memory().numpy()
+    mass = torch.tensor(s.m).pin_memory().numpy()
+    sk.evolve_host(state, mass, s.dt, order, nsteps)
+    got = ics.from_soa(state)
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
