@@ -21,6 +21,7 @@
 #include "kepler_df64.cuh"
 #include "kepler_fp32.cuh"
 #include "kepler_fp64.cuh"
+#include "kepler_weak32.cuh"
 #include "pair_batch_fp64.cuh"
 #include "step_common.cuh"
 #include "step_grp.cuh"
@@ -227,24 +228,130 @@ __global__ void __launch_bounds__(WARPS * 32)
 // particle per tile segment in the earlier contiguous-range kernel (369 MB).
 //
 // The class rule is symmetric in (i, j) (float negation and round-to-nearest
-// are), so one decision serves both ordered pairs.  An FP32-class pair's
-// increments m_j d and -m_i d (float products, formed exactly by two_prod)
-// are summed in double-word form within the window (at most 32 terms per
-// accumulator and phase, exact to 2^-48); the block's column reduction and
-// the row partials go out in FP64, where the apply kernel adds them.  Every
-// other pair joins the warp's FP64 queue, solved 32 at a time and drained at
-// the end of each window, so every queued pair belongs to the current
-// window (drained at every phase, the lone-lane solves before each barrier
-// cost 12 % on GB300).
+// are), so one decision serves both ordered pairs.  An FP32-class pair that
+// moves little (kepler_weak32.cuh: all but 2 in 10^5 of the black-hole
+// cluster's at 16384 bodies, 1 in 10^4 of a 4000-body Plummer sphere's at
+// step 2^-8) takes the direct solve, 66 floating-point instructions without
+// a loop; the iteration and the FP64 queue run for a warp's step only when a
+// lane needs them.  The increments m_j d and -m_i d (float products, formed
+// exactly by two_prod) are summed in double-word form: the leading parts'
+// rounding errors are exact and gather in the second float, which is
+// renormalised every phase (at most 32 terms, 2^-43 of the sum).  The block's
+// column reduction and the row partials go out in FP64, where the apply
+// kernel adds them.  Every other pair joins the warp's FP64 queue, solved 32
+// at a time and drained at the end of each window, so every queued pair
+// belongs to the current window (drained at every phase, the lone-lane solves
+// before each barrier cost 12 % on GB300).
+//
+// What bounds it: the issue rate.  A pair takes 350 warp instructions in 32
+// lanes, 226 of them floating point (12 exact products and double-word sums
+// 120, class and Kepler input 36, solve 66), at 0.66 per cycle and scheduler
+// with 16 warps per SM (128 registers).  Black-hole cluster, 16384 bodies:
+// 2.056 ms per step with the iteration for every pair and sums renormalised
+// at every term, 1.763 with the direct solve, 1.690 with the sums renormalised
+// per phase, 1.566 with the rest of the loop free of 64-bit indices and
+// branches.  24 warps per SM (80 registers, windows of 2 phases) 1.70; windows
+// of 2 phases 1.66; two steps unrolled 1.59.
 
 // SEED: the FP64-class pairs start their FP64 iteration from the root of a
 // single-precision solve of the same pair and finish by the Taylor carry, as
 // in the symmetric FP64 kernel (step_sym.cu); otherwise from a.guess.
 constexpr int kGrpWarps = kMixedGrpWarps;
 
+// acc += p without renormalisation: the leading float's errors are exact and
+// gather in acc.l, which stays below 32 units of its last place over the 32
+// terms that pass between two renormalisations
+__device__ __forceinline__ void dw_acc_raw(dw &acc, dw p)
+{
+    const dw s = two_sum(acc.h, p.h);
+    acc.h = s.h;
+    acc.l = fadd(acc.l, fadd(s.l, p.l));
+}
+
+// The general FP32 solve, out of line: one pair in a thousand or fewer.
+struct Inc32 {
+    float d[6];
+    int iters;
+    bool ok;
+};
+__device__ __noinline__ void pair32_general(const Pair32 &pr, float tau, float post, int guess,
+                                            Inc32 &o)
+{
+    o.ok = pair32_solve(pr, tau, post, guess, o.d, o.iters);
+}
+
+struct QueueCount {
+    int iters, fb, carried;
+    unsigned status;
+};
+
+// FP64 solve of up to 32 queued pairs, one per lane; the twelve products
+// m_j d, -m_i d as double-words to out[lane].
+template <bool SEED>
+__device__ __forceinline__ QueueCount mixed_queue_solve(const StepArgs &a, const float *X32,
+                                                        bool vq, int64_t iq, int64_t jq,
+                                                        float2 (*out)[12])
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t n = a.n;
+    const KeplerParams kp{a.tol, a.max_iter, a.bisection};
+    PairSolve ps;
+    double miq = 0.0, mjq = 0.0;
+    if (vq) {
+        const double *X = a.X;
+        miq = X[6 * n + iq];
+        mjq = X[6 * n + jq];
+        pair_setup(ps, a.tau, miq + mjq, X[iq] - X[jq], X[n + iq] - X[n + jq],
+                   X[2 * n + iq] - X[2 * n + jq], X[3 * n + iq] - X[3 * n + jq],
+                   X[4 * n + iq] - X[4 * n + jq], X[5 * n + iq] - X[5 * n + jq], a.pre,
+                   SEED ? -1 : a.guess);
+        if (SEED) {
+            // the root of the single-precision solve of the pair (unless
+            // t was reduced modulo the period), else the second-order guess
+            float dr[3], dv[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                dr[q] = __fadd_rn(__fsub_rn(X32[q * n + iq], X32[q * n + jq]),
+                                  __fsub_rn(X32[(3 + q) * n + iq], X32[(3 + q) * n + jq]));
+                dv[q] = __fsub_rn(X32[(6 + q) * n + iq], X32[(6 + q) * n + jq]);
+            }
+            const K32 o = k32_phase1(dr, dv, X32[9 * n + iq] + X32[9 * n + jq], a.ptau32,
+                                     a.t32, 2);
+            if (o.ok && __double_as_longlong(ps.t) == __double_as_longlong(a.tau) &&
+                !ps.done) {
+                ps.s = f2d(o.s);
+            } else if (!ps.done) {
+                ps.s = ps.t * ps.ir0;
+                const double cq = 0.5 * ps.s * (ps.eta0 * ps.ir0);
+                if (magbits(cq) < 0x3fe0000000000000LL) ps.s = fma(-cq, ps.s, ps.s);
+            }
+        }
+    } else {
+        ps.done = true;
+        ps.beta = ps.s = 0.0;
+        ps.iters = 0;
+        ps.status = 0;
+    }
+    double d[6];
+    int iters = 0, fb = 0;
+    fp64_solve_warp<SEED>(ps, vq, a.tau, a.post * a.tau, kp, d, iters, fb);
+    if (vq) {
+        // converted to double-words here, with every lane active
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const double xr = mjq * d[q], xc = -miq * d[q];
+            const float rh = __double2float_rn(xr), ch = __double2float_rn(xc);
+            out[lane][q] = make_float2(rh, __double2float_rn(xr - (double)rh));
+            out[lane][6 + q] = make_float2(ch, __double2float_rn(xc - (double)ch));
+        }
+    }
+    return {iters, fb, (vq && ps.carried) ? 1 : 0, vq ? ps.status : 0u};
+}
+
 template <bool STATS, bool SEED>
 __global__ void __launch_bounds__(kGrpWarps * 32, 2)
-    pair_step_grp_mixed_kernel(StepArgs a, MixedArgs ma, GrpLayout L, GrpParts parts)
+    pair_step_grp_mixed_kernel(const __grid_constant__ StepArgs a, MixedArgs ma, GrpLayout L,
+                               GrpParts parts)
 {
     // dynamic shared memory (grp_smem_bytes): the warps' column sums of the
     // window, float4 q2 of column block slot cb holding components 2 q2 and
@@ -327,64 +434,15 @@ __global__ void __launch_bounds__(kGrpWarps * 32, 2)
     // owners' sums and to the warp's column accumulators of the window
     auto flush = [&](int64_t Jw, int cnt) {
         const bool vq = lane < cnt;
-        const int64_t iq = vq ? qi[lane] : 0, jq = vq ? qj[lane] : 0;
-        PairSolve ps;
-        double miq = 0.0, mjq = 0.0;
-        if (vq) {
-            const double *X = a.X;
-            miq = X[6 * n + iq];
-            mjq = X[6 * n + jq];
-            pair_setup(ps, a.tau, miq + mjq, X[iq] - X[jq], X[n + iq] - X[n + jq],
-                       X[2 * n + iq] - X[2 * n + jq], X[3 * n + iq] - X[3 * n + jq],
-                       X[4 * n + iq] - X[4 * n + jq], X[5 * n + iq] - X[5 * n + jq], a.pre,
-                       SEED ? -1 : a.guess);
-            if (SEED) {
-                // the root of the single-precision solve of the pair (unless
-                // t was reduced modulo the period), else the second-order guess
-                float dr[3], dv[3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    dr[q] = __fadd_rn(__fsub_rn(X32[q * n + iq], X32[q * n + jq]),
-                                      __fsub_rn(X32[(3 + q) * n + iq], X32[(3 + q) * n + jq]));
-                    dv[q] = __fsub_rn(X32[(6 + q) * n + iq], X32[(6 + q) * n + jq]);
-                }
-                const K32 o = k32_phase1(dr, dv, X32[9 * n + iq] + X32[9 * n + jq], a.ptau32,
-                                         a.t32, 2);
-                if (o.ok && __double_as_longlong(ps.t) == __double_as_longlong(a.tau) &&
-                    !ps.done) {
-                    ps.s = f2d(o.s);
-                } else if (!ps.done) {
-                    ps.s = ps.t * ps.ir0;
-                    const double cq = 0.5 * ps.s * (ps.eta0 * ps.ir0);
-                    if (magbits(cq) < 0x3fe0000000000000LL) ps.s = fma(-cq, ps.s, ps.s);
-                }
-            }
-        } else {
-            ps.done = true;
-            ps.beta = ps.s = 0.0;
-            ps.iters = 0;
-            ps.status = 0;
-        }
-        double d[6];
-        int iters = 0, fb = 0;
-        fp64_solve_warp<SEED>(ps, vq, a.tau, a.post * a.tau, kp, d, iters, fb);
-        if (vq) {
-            status |= ps.status;
-            // converted to double-words here, with every lane active
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                const double xr = mjq * d[q], xc = -miq * d[q];
-                const float rh = __double2float_rn(xr), ch = __double2float_rn(xc);
-                qres[wib][lane][q] = make_float2(rh, __double2float_rn(xr - (double)rh));
-                qres[wib][lane][6 + q] = make_float2(ch, __double2float_rn(xc - (double)ch));
-            }
-        }
+        const QueueCount qc =
+            mixed_queue_solve<SEED>(a, X32, vq, vq ? qi[lane] : 0, vq ? qj[lane] : 0, qres[wib]);
+        status |= qc.status;
         if (STATS) {
-            carries += (vq && ps.carried) ? 1 : 0;
-            it_sum += iters;
-            fallbacks += fb;
-            it_max = max(it_max, iters);
-            const int wmax = __reduce_max_sync(0xffffffffu, iters);
+            carries += qc.carried;
+            it_sum += qc.iters;
+            fallbacks += qc.fb;
+            it_max = max(it_max, qc.iters);
+            const int wmax = __reduce_max_sync(0xffffffffu, qc.iters);
             if (lane == 0) slots += 32LL * wmax;
         }
         __syncwarp();
@@ -445,38 +503,72 @@ __global__ void __launch_bounds__(kGrpWarps * 32, 2)
             const int64_t Jt = J + cb;
             if (!(I <= Jt && I < nb)) continue;  // warp-uniform: no tile (I, Jt)
             const bool diag = I == Jt;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) racc[q] = fast_two_sum(racc[q].h, racc[q].l);
+            const int i32 = (int)i, j0 = (int)(32 * Jt), n32b = (int)n;
+            // the diagonal tile keeps row sums only: its column products are 0
+            const float mcol = diag ? 0.0f : -mfi;
+            // bit k: this lane has a pair at step k
+            unsigned vmask = 0xffffffffu;
+            if (diag || 32 * I + 32 > n || 32 * Jt + 32 > n) {
+                // columns 0 .. cols - 1, rotated to the lane's first column
+                const int cols = min(32, n32b - j0);
+                const unsigned m = (0xffffffffu >> (32 - cols)) & ~(diag ? 1u << lane : 0u);
+                vmask = irow ? __funnelshift_r(m, m, lane) : 0u;
+            }
+            const float4(*col)[32] = cx[buf][cb];
+            float4(*ca)[32] = cacc[wib][cb];
+#pragma unroll 1
             for (int k = 0; k < 32; ++k) {
                 const int c = (lane + k) & 31;
-                const int64_t j = 32 * Jt + c;
-                const bool valid = irow && j < n && (!diag || c != lane);
-                bool solved32 = false;
-                int it32 = 0;
-                if (valid) {
-                    const float4 c0 = cx[buf][cb][0][c], c1 = cx[buf][cb][1][c],
-                                 c2 = cx[buf][cb][2][c];
-                    const float hi_j[3] = {c0.x, c0.y, c0.z}, lo_j[3] = {c1.x, c1.y, c1.z},
-                                v_j[3] = {c2.x, c2.y, c2.z};
-                    const float mfj = c0.w;
-                    Pair32 pr;
-                    pair32_setup(pr, hi_i, lo_i, v_i, mfi, hi_j, lo_j, v_j, mfj, ma.rule);
-                    if (pr.fp32) {
-                        float d[6];
-                        solved32 = pair32_solve(pr, ma.tau32, ma.post32, a.guess, d, it32);
+                const float4 c0 = col[0][c], c1 = col[1][c], c2 = col[2][c];
+                const float hi_j[3] = {c0.x, c0.y, c0.z}, lo_j[3] = {c1.x, c1.y, c1.z},
+                            v_j[3] = {c2.x, c2.y, c2.z};
+                const float mfj = c0.w;
+                Pair32 pr;
+                pair32_setup(pr, hi_i, lo_i, v_i, mfi, hi_j, lo_j, v_j, mfj, ma.rule);
+                float d[6];
+                const float x[3] = {pr.x0, pr.y0, pr.z0}, v[3] = {pr.vx, pr.vy, pr.vz};
+                const bool weak = pair32_weak(x, v, pr.r2, pr.v2, pr.eta, pr.m, rsqrtf(pr.r2),
+                                              ma.tau32, ma.post32, d);
+                const bool valid = (vmask >> k) & 1u;
+                auto add = [&]() {
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) dw_acc_raw(racc[q], two_prod(mfj, d[q]));
+#pragma unroll
+                    for (int q2 = 0; q2 < 3; ++q2) {
+                        const float4 y = ca[q2][c];
+                        dw a0{y.x, y.y}, a1{y.z, y.w};
+                        dw_acc_raw(a0, two_prod(mcol, d[2 * q2]));
+                        dw_acc_raw(a1, two_prod(mcol, d[2 * q2 + 1]));
+                        ca[q2][c] = make_float4(a0.h, a0.l, a1.h, a1.l);
+                    }
+                };
+                bool solved32 = valid && pr.fp32 && weak;
+                int it32 = 1;
+                if (solved32) add();
+                const unsigned rest = __ballot_sync(0xffffffffu, valid && !solved32);
+                if (rest) {
+                    // the general FP32 solve, or the warp's FP64 queue
+                    if (valid && !solved32 && pr.fp32) {
+                        const Pair32 pc = pr;
+                        Inc32 o;
+                        pair32_general(pc, ma.tau32, ma.post32, a.guess, o);
+                        solved32 = o.ok;
+                        it32 = o.iters;
                         if (solved32) {
 #pragma unroll
-                            for (int q = 0; q < 6; ++q) dw_acc(racc[q], two_prod(mfj, d[q]));
-                            if (!diag) {
-#pragma unroll
-                                for (int q2 = 0; q2 < 3; ++q2) {
-                                    const float4 x = cacc[wib][cb][q2][c];
-                                    dw a0{x.x, x.y}, a1{x.z, x.w};
-                                    dw_acc(a0, two_prod(-mfi, d[2 * q2]));
-                                    dw_acc(a1, two_prod(-mfi, d[2 * q2 + 1]));
-                                    cacc[wib][cb][q2][c] = make_float4(a0.h, a0.l, a1.h, a1.l);
-                                }
-                            }
+                            for (int q = 0; q < 6; ++q) d[q] = o.d[q];
+                            add();
                         }
                     }
+                    const bool need64 = valid && !solved32;
+                    const unsigned mask = __ballot_sync(0xffffffffu, need64);
+                    if (need64) {
+                        qi[tail + __popc(mask & lt_mask)] = i32;
+                        qj[tail + __popc(mask & lt_mask)] = j0 + c;
+                    }
+                    tail += __popc(mask);
                 }
                 if (STATS) {
                     n32 += solved32 ? (diag ? 1 : 2) : 0;  // in ordered pairs
@@ -487,13 +579,6 @@ __global__ void __launch_bounds__(kGrpWarps * 32, 2)
                     const int wmax = __reduce_max_sync(0xffffffffu, its);
                     if (lane == 0) slots += 32LL * wmax;
                 }
-                const bool need64 = valid && !solved32;
-                const unsigned mask = __ballot_sync(0xffffffffu, need64);
-                if (need64) {
-                    qi[tail + __popc(mask & lt_mask)] = (int)i;
-                    qj[tail + __popc(mask & lt_mask)] = (int)j;
-                }
-                tail += __popc(mask);
                 __syncwarp();
                 if (tail >= 32) {
                     flush(J, 32);
