@@ -101,14 +101,14 @@ extern "C" {
                                       partials per segment: up to 12 n^2 bytes of
                                       scratch), the FP64 default below 4096
                                       bodies (the mixed form's under the literal
-                                      rule too; the double-word form's up to about
-                                      13400)                                       */
+                                      rule too, its other rule's up to 640; the
+                                      double-word form's up to about 13400)        */
 #define SAKURA_FLAG_GROUPS 64u     /* symmetric FP64 and mixed steps: always the
                                       row-group kernel (blocks of warps sweep column
                                       blocks together, column sums reduced per
                                       block: about n^2 / 2.7 bytes), the default
                                       beyond, and the mixed form's under
-                                      SAKURA_MIXED_RULE_HYP                        */
+                                      SAKURA_MIXED_RULE_HYP above 640 bodies       */
 
 #define SAKURA_BATCH_MAX_N 64     /* largest system of sakura_step_batched       */
 
@@ -194,10 +194,11 @@ int sakura_set_stream(void *stream);
  * whose partial sums take up to 8 x 6 x 8 ceil(n/32) n bytes of library
  * scratch (12 MB at n = 1024), below 4096 bodies, and in row-group phases
  * from there, whose partials take about n^2 / 2.7 bytes (0.1 GB at 16384);
- * the mixed form uses row groups under SAKURA_MIXED_RULE_HYP, and under the
- * literal rule the FP64 kernel of its size with an inline class test
- * (SAKURA_FLAG_TILES / SAKURA_FLAG_GROUPS force either kernel).  Where the symmetric scratch
- * would pass 16 GB the ordered kernel is used.  Systems of 2 <= n <= 20 in the
+ * the mixed form uses row groups of its own under SAKURA_MIXED_RULE_HYP above
+ * 640 bodies, and below, and under the literal rule, the FP64 kernel of its
+ * size with an inline class test (SAKURA_FLAG_TILES / SAKURA_FLAG_GROUPS force
+ * either kernel).  Where the symmetric scratch would pass 16 GB the ordered
+ * kernel is used.  Systems of 2 <= n <= 20 in the
  * FP64 form with symmetric pairs and a non-learned guess run in one launch
  * of a single-block kernel that keeps the system in shared memory and packs
  * the pairs densely over its lanes (no scratch; SAKURA_FLAG_NO_SMALL turns

@@ -313,9 +313,16 @@ bool fp64_groups(int64_t n)
 // The mixed form's kernels.  Under the literal rule, which admits few pairs
 // in clusters (the black-hole cluster: 0.01 % of them), the FP64 kernels
 // with an inline class test: on tiles (step_sym.cu) or in row groups
-// (step_grp.cu) as for the FP64 form.  Under the hyperbolic rule the
-// row-group mixed kernel (step_mixed.cu), or the tile kernel with the inline
-// test when SAKURA_FLAG_TILES forces it.
+// (step_grp.cu) as for the FP64 form.  Under the hyperbolic rule the tile
+// kernel with the inline test up to kMixedTilesMaxN bodies, where a row
+// group's warps run the few tiles there are, and their FP64 pairs, one after
+// the other, and the row-group mixed kernel (step_mixed.cu) beyond.  Four
+// steps of a run in us, row groups / tiles, Plummer spheres and (in brackets)
+// stars around a heavy black hole: 64 bodies 550 / 80 (148 / 77), 256 320 / 90
+// (172 / 86), 512 222 / 160 (189 / 126), 640 214 / 199 (189 / 174), 700 214 /
+// 216 (189 / 180); two steps of 760 bodies 108 / 129 (98 / 110).  The flags
+// force either kernel.
+constexpr int64_t kMixedTilesMaxN = 640;
 enum class MixedKernel { Tiles, Fp64Groups, MixedGroups };
 
 MixedKernel mixed_kernel(int64_t n)
@@ -323,6 +330,7 @@ MixedKernel mixed_kernel(int64_t n)
     if (g.cfg.mixed_rule == SAKURA_MIXED_RULE_LITERAL)
         return fp64_groups(n) ? MixedKernel::Fp64Groups : MixedKernel::Tiles;
     if (g.cfg.flags & SAKURA_FLAG_TILES) return MixedKernel::Tiles;
+    if (!(g.cfg.flags & SAKURA_FLAG_GROUPS) && n <= kMixedTilesMaxN) return MixedKernel::Tiles;
     return MixedKernel::MixedGroups;
 }
 
@@ -574,6 +582,13 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
     const int64_t T = tiles * 32;
     int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks : (int64_t)g.sm_count * bps;
     blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, T / 4));
+    // mixed form: two tile-steps per warp where one would take more than one
+    // block per SM and two take at most two (256 bodies, four steps: 89 us
+    // against 107; 333: 108 against 126; outside that range one is faster:
+    // 128 bodies 80 against 89)
+    if (mixed && !weak && g.cfg.grid_blocks <= 0 && T / 4 > g.sm_count &&
+        T / 8 <= 2 * (int64_t)g.sm_count)
+        blocks = T / 8;
     const int64_t W = blocks * 4;
     const int Smax = (int)((32 * W + T - 1) / T + 1);
     const int64_t nslots = nb * Smax;
@@ -653,7 +668,7 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
                                   g.stream);
     else
         sakura::launch_apply_sym(dst, X, X32, rows, partial, n, Smax, W, T, post_drift,
-                                 fuse && !mixed, next_drift, g.d_status, g.stream);
+                                 fuse, next_drift, g.d_status, g.stream);
     rc = launch_error();
     if (rc) return rc;
     g.steps += 1;
@@ -783,12 +798,14 @@ int step_weak_small(const double *src, double *dst, const double *masses, int64_
 }
 
 // Sub-steps whose apply kernel can also drift for the next one: the FP64
-// form's symmetric kernels, and the double-word form's weak ones.
+// form's symmetric kernels, the double-word form's weak ones and the mixed
+// form's tiles.
 bool fusable(int64_t n, int order, double tau)
 {
     return sym_path(n) &&
            (g.cfg.precision == SAKURA_PREC_FP64 ||
-            (g.cfg.precision == SAKURA_PREC_DF64 && weak_form(order, tau)));
+            (g.cfg.precision == SAKURA_PREC_DF64 && weak_form(order, tau)) ||
+            (g.cfg.precision == SAKURA_PREC_MIXED && mixed_kernel(n) == MixedKernel::Tiles));
 }
 
 int step_device(const double *src, double *dst, const double *masses, int64_t n, double dt,

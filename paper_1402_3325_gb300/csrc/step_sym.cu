@@ -25,6 +25,7 @@
 
 #include "kepler_df64.cuh"
 #include "kepler_fp64.cuh"
+#include "kepler_weak32.cuh"
 #include "mlp_infer.cuh"
 #include "pair_batch_fp64.cuh"
 #include "step_common.cuh"
@@ -133,7 +134,11 @@ __global__ void __launch_bounds__(128, MIXED ? 2 : ((SEED || LEARNED) ? 3 : 4))
                                  a.rule);
                     if (pr.fp32) {
                         int it32 = 0;
-                        lane32 = pair32_solve(pr, a.t32, a.post32, a.guess, d32, it32);
+                        const float xx[3] = {pr.x0, pr.y0, pr.z0}, vv[3] = {pr.vx, pr.vy, pr.vz};
+                        lane32 = pair32_weak(xx, vv, pr.r2, pr.v2, pr.eta, pr.m, rsqrtf(pr.r2),
+                                             a.t32, a.post32, d32);
+                        if (!lane32)
+                            lane32 = pair32_solve(pr, a.t32, a.post32, a.guess, d32, it32);
                     }
                 }
                 if (!lane32)
