@@ -101,7 +101,18 @@ EMU_CARRY_MULS = 4
 EMU_ITER_MULS = 10
 
 
+# a weakly perturbed pair (csrc/kepler_weak.cuh), which nearly every pair of
+# these workloads is: FP64 separation 3, r0^2 5, 1 - r0^2 y^2 2, the leading
+# factor 3, its products with the two masses 2 (on the integer pipes) and the
+# two velocity sums 12.  Its corrections, in double-word FP32 arithmetic, and
+# the FP64 solves of the other pairs are not counted.
+C_WEAK = 27
+EMU_WEAK_MULS = 2
+
+
 def _integer_pipe_flops(kernel, guess, kbar, mixed=False):
+    if kernel in ("pair_step_grp_weak", "pair_step_weak"):
+        return EMU_WEAK_MULS
     if kernel not in ("pair_step_grp", "pair_step_sym", "batched"):
         return 0
     if mixed:  # the inline class test: row groups only
@@ -114,8 +125,7 @@ def _integer_pipe_flops(kernel, guess, kbar, mixed=False):
 
 
 # FP32-class pair of the symmetric mixed form (see the roofline code below)
-C_MIX32_FIX = 44 + 44 + 168
-C_MIX32_ITER = 71
+C_MIX32 = 44 + 99 + 132
 
 # FP64 ALU peak of one GB300: 152 SMs x 2 FP64 FMA units x 2 flop x 2.07 GHz
 # (the unit count follows from the nominal 1.25 TFLOP/s at 2.07 GHz).
@@ -236,6 +246,7 @@ KERNEL_SOURCES = {"pair_step_sym": "step_sym.cu", "pair_step_grp": "step_grp.cu"
                   "pair_step_fp64": "step_fp64.cu", "pair_step_sym_df64": "step_df64.cu",
                   "pair_step_grp_df64": "step_df64.cu",
                   "pair_step_grp_mixed": "step_mixed.cu", "pair_step_mixed": "step_mixed.cu",
+                  "pair_step_weak": "step_weak.cu", "pair_step_grp_weak": "step_weak.cu",
                   "small": "step_small.cu", "batched": "step_batched.cu"}
 
 
@@ -639,7 +650,17 @@ def _roofline(workload, form, pairs, guess, n, small, m):
     fp64_peak_src = ("152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (derived from the nominal"
                      " 1.25 TFLOP/s; an FP64 FMA probe on this GPU sustains 1.06 TFLOP/s)")
     fp32_peak_src = "152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz"
-    if form == "df64":
+    # the order-2 steps whose weakly perturbed pairs take the short solve
+    weak = (not small and pairs == "symmetric" and
+            (form in ("fp64", "df64") or (form == "mixed" and share < 0.5 and guess == "fp32")))
+    if weak:
+        flops = C_WEAK
+        peak, pipe, src = FP64_PEAK_GFLOPS / 1e3, "fp64", fp64_peak_src + (
+            "; flops of the FP64 part of a weakly perturbed pair, counted by hand: the corrections"
+            " on the FP32 pipe, which issue most instructions, and the other pairs' FP64 solves"
+            " are not counted")
+        kname = "pair_step_grp_weak" if m["row_groups"] else "pair_step_weak"
+    elif form == "df64":
         flops = DF64_FLOPS_PER_SOLVE.get(workload)
         peak, pipe, src = FP32_PEAK_GFLOPS / 1e3, "fp32", fp32_peak_src + (
             "; flops per solve counted by running the double-word code on the host with an"
@@ -647,14 +668,11 @@ def _roofline(workload, form, pairs, guess, n, small, m):
         kname = "small" if small else (
             "pair_step_grp_df64" if m["row_groups"] else "pair_step_sym_df64")
     elif form == "mixed" and pairs == "symmetric" and share >= 0.5:
-        # FP32 flops of an FP32-class unordered pair (hand count from
-        # csrc/kepler_fp32.cuh and csrc/step_mixed.cu, FMA = 2): class test
-        # 44, solve setup 12, epilogue with increments and finiteness test
-        # 32, per Laguerre iteration 71 (evaluation 37, step 9, stopping
-        # test 2, carry of G1..G3 and F' 23), double-word sums of m_j d and
-        # -m_i d 168 (12 x (two_prod 3 + renormalised sum 11)); kbar =
-        # single-precision iterations per solve
-        flops = share * (C_MIX32_FIX + kbar * C_MIX32_ITER)
+        # FP32 flops of an FP32-class unordered pair that moves little (nearly
+        # all; hand count from csrc/kepler_weak32.cuh and csrc/step_mixed.cu,
+        # FMA = 2): class test and Kepler input 44, direct solve 99,
+        # double-word sums of m_j d and -m_i d 132 (12 x (two_prod 3 + sum 8))
+        flops = share * C_MIX32
         peak, pipe, src = FP32_PEAK_GFLOPS / 1e3, "fp32", fp32_peak_src + "; flops counted by hand"
         kname = "pair_step_grp_mixed" if m["row_groups"] else "pair_step_sym"
     elif form == "mixed" and pairs == "symmetric":
