@@ -285,7 +285,8 @@ def _profiled_traffic(workload: str, kernel: str):
             if ":" in ln and ln.lstrip().startswith("- "):
                 k, v = ln.lstrip()[2:].split(":", 1)
                 vals[k.strip()] = v.strip().strip("`")
-    if vals.get("kernel_sources_sha256_16") != _kernel_sources_hash(kernel):
+    taken = vals.get("sources_sha256_16", vals.get("kernel_sources_sha256_16"))
+    if taken != _kernel_sources_hash(kernel):
         return None
     try:
         return float(vals["dram_bytes_per_launch"])

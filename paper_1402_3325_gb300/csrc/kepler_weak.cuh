@@ -6,7 +6,7 @@
 // FP64 instructions per pair and its kernels are bound by them.  Most pairs
 // of a step move by a small part of their separation.  For those the map is
 // a known leading term plus corrections, and only the leading term needs
-// FP64 arithmetic: 19 FP64 instructions per pair, the corrections in
+// FP64 arithmetic: 15 FP64 instructions per pair, the corrections in
 // double-word FP32 arithmetic (df64.cuh).
 //
 // In the units r0 (separation) and t (step), with x, w = t v the relative

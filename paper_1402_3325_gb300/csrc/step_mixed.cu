@@ -243,10 +243,10 @@ __global__ void __launch_bounds__(WARPS * 32)
 // belongs to the current window (drained at every phase, the lone-lane solves
 // before each barrier cost 12 % on GB300).
 //
-// What bounds it: the issue rate.  A pair takes 350 warp instructions in 32
-// lanes, 226 of them floating point (12 exact products and double-word sums
-// 120, class and Kepler input 36, solve 66), at 0.66 per cycle and scheduler
-// with 16 warps per SM (128 registers).  Black-hole cluster, 16384 bodies:
+// What bounds it: the issue rate.  A pair takes 331 warp instructions in 32
+// lanes, 223 of them floating point (12 exact products and double-word sums
+// 120, class and Kepler input 36, solve 66), at 0.73 per cycle and scheduler
+// with 16 warps per SM (128 registers; ncu, 8192 bodies).  Black-hole cluster, 16384 bodies:
 // 2.056 ms per step with the iteration for every pair and sums renormalised
 // at every term, 1.763 with the direct solve, 1.690 with the sums renormalised
 // per phase, 1.566 with the rest of the loop free of 64-bit indices and

@@ -12,17 +12,17 @@
 // 75-instruction FP64 solve for one lane; a step with more than
 // kWeakInline strong lanes solves them at once.
 //
-// Bound: the FP64 pipe (18 FP64 instructions per pair and 16 cycles each)
-// and the issue slots (about 930 instructions per pair) nearly alike: ncu at
-// 4000 bodies, 81 % and 55 % before three FP64 instructions more were taken
-// out.  ms per step: 16384 bodies (black hole) 20.36 -> 5.18 in row groups,
-// 5.12 on tiles; Plummer 1024 0.109 -> 0.044, 2048 0.358 -> 0.106, 4000
-// 1.30 -> 0.352 (the kernels of step_sym.cu and step_grp.cu with the seed
-// before); the double-word form, 16384 bodies with binaries: 8.29 -> 5.37
-// (step_df64.cu before: every pair in 1922 double-word flops); the mixed
-// form's literal rule, 5003 bodies: 2.11 -> 0.56; the default guess, 2999
-// bodies, a fourth-order step on host arrays: 3.26 -> 0.75; the learned
-// guess, 8192 bodies with binaries: 7.07 -> 1.58.
+// Bound: the FP64 pipe (16 FP64 instructions per pair and 16 cycles each)
+// and the issue slots (950 instructions per pair and warp) nearly alike: ncu
+// at 8192 bodies (black hole), 67 % and 63 %, neither full with the 12 warps
+// per SM that 168 registers leave.  ms per step: 16384 bodies (black hole)
+// 20.36 -> 5.08 in row groups; Plummer 1024 0.109 -> 0.043, 2048 0.358 ->
+// 0.103, 4000 1.30 -> 0.332 (the kernels of step_sym.cu and step_grp.cu with
+// the seed before); the double-word form, 16384 bodies with binaries: 8.29 ->
+// 5.45 (step_df64.cu before: every pair in 1922 double-word flops); the mixed
+// form's literal rule, 5003 bodies: 2.11 -> 0.55; the default guess, 2999
+// bodies, a fourth-order step on host arrays: 3.26 -> 0.74; the learned
+// guess, 8192 bodies with binaries: 7.06 -> 1.55.
 #include <cuda_runtime.h>
 
 #include "kepler_df64.cuh"
