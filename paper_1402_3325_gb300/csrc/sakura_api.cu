@@ -301,7 +301,12 @@ double group_partial_bytes(int64_t n, int G)
 // 0.412, + 4095 stars 1.376 / 1.351, + 8191 stars 5.378 / 5.182, + 12287
 // stars 12.07 / 11.54, + 16383 stars 21.58 / 20.41; Plummer 2048 bodies
 // 0.358 / 0.393, 4096 1.354 / 1.357, 8192 5.350 / 5.262, 12288 12.02 /
-// 11.71, 16384 21.47 / 20.73).  The flags force either kernel.
+// 11.71, 16384 21.47 / 20.73).  The kernels of the weak pairs take the same
+// line, though with them the tiles are the faster side at every size (us per
+// step, tiles / row groups: 2048 bodies 104 / 120, 4096 354 / 365, 8192 1294 /
+// 1357, 16384 5137 / 5288): from 4096 bodies the row groups' partials are a
+// fifth to a seventh of the tiles' scratch (0.1 against 0.8 GB at 16384) and
+// stay in L2.  The flags force either kernel.
 constexpr int64_t kFp64GroupsMinN = 4096;
 bool fp64_groups(int64_t n)
 {
