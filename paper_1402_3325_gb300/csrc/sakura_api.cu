@@ -363,6 +363,8 @@ bool df64_groups(int64_t n)
 //   - the mixed form with the seed under the literal rule with e_max < 1,
 //     where only bound pairs are FP32-class: few in a cluster, and told from
 //     the others by their energy.
+// Of one run's sub-steps either all take it or none (weak_run): the scratch,
+// which holds the run's copy of the masses, then has one size throughout.
 bool weak_form(int order, double tau)
 {
     if (order != 2 || !(std::fabs(tau) >= 1e-18 && std::fabs(tau) <= 1e18)) return false;
@@ -372,6 +374,14 @@ bool weak_form(int order, double tau)
         return seed && g.cfg.mixed_rule == SAKURA_MIXED_RULE_LITERAL && g.cfg.mixed_e_max < 1.0;
     return seed || (!(g.cfg.flags & SAKURA_FLAG_STATS) && g.cfg.kepler_max_iter >= 8 &&
                     g.cfg.kepler_tol >= 1.0);
+}
+
+// Whether the sub-steps w[0] dt .. w[cnt - 1] dt of a run are weak steps.
+bool weak_run(int order, double dt, const double *w, int cnt)
+{
+    for (int k = 0; k < cnt; ++k)
+        if (!weak_form(order, w[k] * dt)) return false;
+    return true;
 }
 
 sakura::WeakForm weak_kind()
@@ -460,14 +470,13 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
 // state, written by the previous apply kernel; fuse: the apply kernel also
 // applies the next sub-step's drift next_drift and writes its X (and X32).
 int step_device_fp64_grp(const double *src, double *dst, const double *masses, int64_t n,
-                         double dt, int order, bool prepped, bool fuse, double next_drift,
-                         bool mixed = false)
+                         double dt, int order, bool weak, bool prepped, bool fuse,
+                         double next_drift, bool mixed = false)
 {
     const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
     const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED &&
                          g.cfg.precision == SAKURA_PREC_FP64;
     const bool seed = g.cfg.guess == SAKURA_GUESS_FP32 && g.cfg.precision != SAKURA_PREC_DF64;
-    const bool weak = weak_form(order, dt);
     int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks
                      : (int64_t)g.sm_count *
                            (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats, weak_kind())
@@ -556,25 +565,26 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
 // by the previous apply kernel (FP64 form only); fuse: the apply kernel also
 // applies the next sub-step's drift next_drift and writes its X (and X32).
 int step_device_sym(const double *src, double *dst, const double *masses, int64_t n, double dt,
-                    int order, bool df64, bool mixed, bool prepped = false, bool fuse = false,
-                    double next_drift = 0.0)
+                    int order, bool df64, bool mixed, bool weak, bool prepped, bool fuse,
+                    double next_drift)
 {
     if (mixed) {
         const MixedKernel k = mixed_kernel(n);
         if (k == MixedKernel::MixedGroups)
             return step_device_mixed_grp(src, dst, masses, n, dt, order);
         if (k == MixedKernel::Fp64Groups)
-            return step_device_fp64_grp(src, dst, masses, n, dt, order, false, false, 0.0, true);
+            return step_device_fp64_grp(src, dst, masses, n, dt, order, weak, false, false, 0.0,
+                                        true);
     }
-    const bool weak = weak_form(order, dt);
     if (df64 && df64_groups(n))
-        return weak ? step_device_fp64_grp(src, dst, masses, n, dt, order, prepped, fuse,
+        return weak ? step_device_fp64_grp(src, dst, masses, n, dt, order, weak, prepped, fuse,
                                            next_drift)
                     : step_device_df64_grp(src, dst, masses, n, dt, order);
     const bool dwf = df64 && weak;  // the double-word form's weak kernel
     df64 = df64 && !weak;
     if (!df64 && !dwf && !mixed && fp64_groups(n))
-        return step_device_fp64_grp(src, dst, masses, n, dt, order, prepped, fuse, next_drift);
+        return step_device_fp64_grp(src, dst, masses, n, dt, order, weak, prepped, fuse,
+                                    next_drift);
     const bool stats = (g.cfg.flags & SAKURA_FLAG_STATS) != 0;
     const bool learned = !df64 && !dwf && !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
     const bool seed = !df64 && !dwf && g.cfg.guess == SAKURA_GUESS_FP32;
@@ -719,9 +729,9 @@ bool sym_path(int64_t n)
 // (2; 4; 8 per warp; the general tile kernel) on 152 SMs: 256 bodies (49; 51;
 // 66; 83), 320 (56; 54; 68; 136), 512 (120; 90; 90; 135), 576 (-; 107; 110;
 // 135), 760 (-; 146; 113; 155), 928 (-; -; 151; 167); 1024 (-; -; 190; 175).
-int weak_small_steps(int64_t n, int order, double tau)
+int weak_small_steps(int64_t n)
 {
-    if (g.cfg.grid_blocks > 0 || !sym_path(n) || !weak_form(order, tau)) return 0;
+    if (g.cfg.grid_blocks > 0 || !sym_path(n)) return 0;
     if (g.cfg.precision == SAKURA_PREC_MIXED ? mixed_kernel(n) != MixedKernel::Tiles
         : g.cfg.precision == SAKURA_PREC_DF64 ? df64_groups(n)
                                               : fp64_groups(n))
@@ -730,15 +740,6 @@ int weak_small_steps(int64_t n, int order, double tau)
     for (int k = 1; k <= 3; ++k)
         if ((tiles * 8 >> k) <= k * (int64_t)g.sm_count) return 1 << k;
     return 0;
-}
-
-// The same for a run whose sub-steps have these time weights.
-int weak_small_run(int64_t n, int order, double dt, const double *w, int cnt)
-{
-    int steps = 0;
-    for (int k = 0; k < cnt; ++k)
-        if (!(steps = weak_small_steps(n, order, w[k] * dt))) return 0;
-    return steps;
 }
 
 // A weak step of a small system (step_weak.cu): pair and apply kernels.
@@ -805,21 +806,22 @@ int step_weak_small(const double *src, double *dst, const double *masses, int64_
 // Sub-steps whose apply kernel can also drift for the next one: the FP64
 // form's symmetric kernels, the double-word form's weak ones and the mixed
 // form's tiles.
-bool fusable(int64_t n, int order, double tau)
+bool fusable(int64_t n, bool weak)
 {
     return sym_path(n) &&
            (g.cfg.precision == SAKURA_PREC_FP64 ||
-            (g.cfg.precision == SAKURA_PREC_DF64 && weak_form(order, tau)) ||
+            (g.cfg.precision == SAKURA_PREC_DF64 && weak) ||
             (g.cfg.precision == SAKURA_PREC_MIXED && mixed_kernel(n) == MixedKernel::Tiles));
 }
 
 int step_device(const double *src, double *dst, const double *masses, int64_t n, double dt,
-                int order, bool prepped = false, bool fuse = false, double next_drift = 0.0)
+                int order, bool weak, bool prepped, bool fuse, double next_drift)
 {
     if (sym_path(n))
         return step_device_sym(src, dst, masses, n, dt, order,
                                g.cfg.precision == SAKURA_PREC_DF64,
-                               g.cfg.precision == SAKURA_PREC_MIXED, prepped, fuse, next_drift);
+                               g.cfg.precision == SAKURA_PREC_MIXED, weak, prepped, fuse,
+                               next_drift);
     const Plan p = plan_step(n);
     const int64_t slots = sakura::pair_step_slots(n, p.W);
     const bool mixed = g.cfg.precision == SAKURA_PREC_MIXED;
@@ -930,10 +932,11 @@ const double *step_masses(int64_t n) { return (const double *)g.partial.ptr + 6 
 // nsteps steps of the given order as one run of sub-steps: the first reads
 // src, the last writes dst, the others read and write mid (src, mid and dst
 // may be the same buffer).  From the second sub-step on, the masses come
-// from the copy that the first drift kernel left in the scratch (same n, so
-// the scratch is not reallocated).  On symmetric FP64 tiles every apply
-// kernel but the last also drifts for the next sub-step, so only the first
-// sub-step runs a prep kernel (the same arithmetic: results are unchanged).
+// from the copy that the first drift kernel left in the scratch, which is not
+// reallocated in between: every sub-step of a run has the same n, options and
+// weak, on which alone its size depends.  Where fusable, every apply kernel
+// but the last also drifts for the next sub-step, so only the first sub-step
+// runs a prep kernel (the same arithmetic: results are unchanged).
 int run_substeps(const double *src, double *mid, double *dst, const double *masses, int64_t n,
                  double dt, int order, int nsteps)
 {
@@ -941,7 +944,8 @@ int run_substeps(const double *src, double *mid, double *dst, const double *mass
     int so;
     const int cnt = substeps(order, w, &so);
     const int64_t total = (int64_t)cnt * nsteps;
-    const int steps = weak_small_run(n, so, dt, w, cnt);
+    const bool weak = weak_run(so, dt, w, cnt);
+    const int steps = weak ? weak_small_steps(n) : 0;
     if (steps > 0) {
         if (src != mid) {  // host memory
             const int rc = grow(g.partial, (size_t)(7 * n + (n + 31) / 32 * (8 / steps) * 6 * n) *
@@ -965,11 +969,10 @@ int run_substeps(const double *src, double *mid, double *dst, const double *mass
         const double t = w[k % cnt] * dt;
         const double tn = last ? 0.0 : w[(k + 1) % cnt] * dt;
         const double next_drift = so == 2 ? 0.5 * tn : (so == 1 ? 0.0 : tn);  // as the prep
-        const bool fuse_k =
-            !last && fusable(n, so, t) && weak_form(so, t) == weak_form(so, tn);
+        const bool fuse_k = !last && fusable(n, weak);
         const int rc = step_device(k == 0 ? src : mid, last ? dst : mid,
-                                   k == 0 ? masses : step_masses(n), n, t, so, prepped, fuse_k,
-                                   next_drift);
+                                   k == 0 ? masses : step_masses(n), n, t, so, weak, prepped,
+                                   fuse_k, next_drift);
         if (rc) return rc;
         prepped = fuse_k;
     }
@@ -1226,7 +1229,8 @@ int sakura_evolve_host(double *state, const double *masses, int64_t n, double dt
         int so;
         double *ds = nullptr;
         const int cnt = substeps(order, w, &so);
-        if ((int64_t)cnt * nsteps > 1 || weak_small_run(n, so, dt, w, cnt) > 0) {
+        if ((int64_t)cnt * nsteps > 1 ||
+            (weak_run(so, dt, w, cnt) && weak_small_steps(n) > 0)) {
             rc = grow(g.host_state, sbytes);
             if (rc) return rc;
             ds = (double *)g.host_state.ptr;
