@@ -9,9 +9,8 @@ from paper_1402_3325_gb300 import ics
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision", [0, 2], ids=["fp64", "df64"])
 @pytest.mark.parametrize("order,dt", [(4, 6.5e-19), (8, 5e-19)])
-def test_composed_step_across_the_smallest_step_size(order, dt, precision):
+def test_composed_step_across_the_smallest_step_size(order, dt):
     # cold, so that the velocities after the step are its increments: 3 and 27
     # sub-steps, each with 1e-13 of its own increments, which are up to 8 times
     # the whole step's; in a fresh context, whose scratch holds nothing else
@@ -20,8 +19,7 @@ def test_composed_step_across_the_smallest_step_size(order, dt, precision):
     s = ics.random_cluster(1000, seed=4)
     s.v[:] = 0.0
     sk.finalize()
-    sk.init(0, stream=torch.cuda.current_stream().cuda_stream, guess=sk.GUESS_FP32,
-            precision=precision)
+    sk.init(0, stream=torch.cuda.current_stream().cuda_stream, guess=sk.GUESS_FP32)
     state, mass = torch.tensor(s.soa(), device="cuda"), torch.tensor(s.m, device="cuda")
     sk.step(state, mass, dt, order)
     sk.check()
