@@ -723,7 +723,8 @@ bool sym_path(int64_t n)
 }
 
 // Tile-steps per warp of the small weak kernel: 2, 4 or 8, the fewest that
-// keep the grid at one, two or three blocks per SM; 0 where it is not used.
+// keep the grid at one, two or three blocks per SM; 0 where it is not used
+// (SAKURA_FLAG_TILES asks for the general tile kernel).
 // More of them lengthen a warp's chain (0.5 us each), fewer make more blocks
 // and partial sums than the SMs take at once.  Four steps of a run in us with
 // (2; 4; 8 per warp; the general tile kernel) on 152 SMs: 256 bodies (49; 51;
@@ -731,7 +732,7 @@ bool sym_path(int64_t n)
 // 135), 760 (-; 146; 113; 155), 928 (-; -; 151; 167); 1024 (-; -; 190; 175).
 int weak_small_steps(int64_t n)
 {
-    if (g.cfg.grid_blocks > 0 || !sym_path(n)) return 0;
+    if (g.cfg.grid_blocks > 0 || (g.cfg.flags & SAKURA_FLAG_TILES) || !sym_path(n)) return 0;
     if (g.cfg.precision == SAKURA_PREC_MIXED ? mixed_kernel(n) != MixedKernel::Tiles
         : g.cfg.precision == SAKURA_PREC_DF64 ? df64_groups(n)
                                               : fp64_groups(n))

@@ -84,3 +84,14 @@ def test_a_run_reads_only_scratch_that_it_holds(fake_library, form, n, host):
             assert log and not [k for k in log if k.endswith("!")], (order, dt, log)
             pair = {k for k in log if re.fullmatch("(grp_|small_)?weak|sym|grp|df64|grp_df64", k)}
             assert len(pair) == 1, (order, dt, pair)
+
+
+@pytest.mark.parametrize("n", [21, 129, 417, 928])
+@pytest.mark.parametrize("form", FORMS)
+def test_the_flags_choose_the_kernel_they_name(fake_library, form, n):
+    for flag, kernel in ((0, "small_weak"), (sk.FLAG_TILES, "weak"), (sk.FLAG_GROUPS, "grp_weak")):
+        if form == "df64" and flag == sk.FLAG_GROUPS:
+            continue  # the flag is for the other two forms
+        with Run(fake_library, pair_mode=sk.PAIRS_SYMMETRIC, flags=flag, **FORMS[form]) as r:
+            log = r.evolve(n, 2.0 ** -8, 2)
+        assert [k for k in log if k.endswith("weak") and not k.startswith("prep")] == [kernel], log
