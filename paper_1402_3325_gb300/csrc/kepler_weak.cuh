@@ -167,10 +167,15 @@ DW_HD double mul_soft(double a, double b)
     return fpb_double((int64_t)(r | ((uint64_t)((ah ^ bh) & 0x80000000u) << 32)));
 }
 
-// h + l as a double; an exact zero stays zero
+// h + l as a double for |h| < 2^63; an exact zero stays zero, and so does the
+// value of a subnormal float (the sums of light pairs end there): the floats
+// are scaled by 2^64 into the normal range, on the FP32 pipe
 DW_HD double dw_to_double(dw x)
 {
-    const double h = widen(x.h), l = widen(x.l);
+    const float hs = fmul(x.h, 0x1p64f), ls = fmul(x.l, 0x1p64f);
+    const int64_t down = 64LL << 52;
+    const double h = fpb_double(fpb_bits(widen(hs)) - down);
+    const double l = fpb_double(fpb_bits(widen(ls)) - down);
     return (x.h != 0.0f ? h : 0.0) + (x.l != 0.0f ? l : 0.0);
 }
 
@@ -312,9 +317,12 @@ DW_HD void weak_acc(dw &acc, dw x, dw y)
 
 // the limits of weak_class, as ratios to r0^2 or plain
 constexpr float kWeakEps2 = 0x1p-10f, kWeakMu = 0x1p-10f, kWeakSpeed2 = 0x1p-8f;
-// smallest tau^2 m / r0^2: the double-words' remainders stay normal floats
-// where they matter
-constexpr float kWeakMin = 1e-28f;
+// Smallest tau^2 m / r0^2 of a particle, and smallest tau^2 m and tau^2 m /
+// r0^3: a float's last place is no smaller than 2^-149, so the increments'
+// double-word sums (of the size of the first times eps r0) are off by up to a
+// few 2^-149, 2^-54 of the increment, and the remainders of the mass and of
+// its product with 1 / r0^3 by 2^-50, times eps.
+constexpr float kWeakMin = 1e-28f, kWeakMinFactor = 0x1p-100f;
 
 // One particle: position before the drift, tau m, and tau v, tau^2 m as
 // double-words.
@@ -353,10 +361,10 @@ DW_HD bool weak_class(const WeakParticle &a, float sa, const WeakParticle &b, We
     d.w2 = ffma(d.w[0].h, d.w[0].h, ffma(d.w[1].h, d.w[1].h, fmul(d.w[2].h, d.w[2].h)));
     d.y = rsqrt_approx(d.r2d.h);
     const float y2 = fmul(d.y, d.y);
-    const float mu = fmul(fmul(fadd(a.mh.h, b.mh.h), d.y), y2);
+    const float mu = fmul(fmul(fadd(a.mh.h, b.mh.h), d.y), y2), mm = fminf(a.mh.h, b.mh.h);
     return hi - 0x3c300000u < 0x07800000u && d.w2 <= fmul(kWeakEps2, d.r2d.h) &&
            fadd(sa, weak_speed2(b)) <= fmul(kWeakSpeed2, d.r2d.h) && mu <= kWeakMu &&
-           fmul(fminf(a.mh.h, b.mh.h), y2) >= kWeakMin;
+           fmul(mm, y2) >= kWeakMin && fmul(mm, fminf(1.0f, fmul(d.y, y2))) >= kWeakMinFactor;
 }
 
 // Whether a class test of e < e_max < 1 on float copies (kepler_fp32.cuh) is
