@@ -6,7 +6,7 @@
 // FP64 instructions per pair and its kernels are bound by them.  Most pairs
 // of a step move by a small part of their separation.  For those the map is
 // a known leading term plus corrections, and only the leading term needs
-// FP64 arithmetic: 15 FP64 instructions per pair, the corrections in
+// FP64 arithmetic: 16 FP64 instructions per pair, the corrections in
 // double-word FP32 arithmetic (df64.cuh).
 //
 // In the units r0 (separation) and t (step), with x, w = t v the relative
@@ -21,7 +21,8 @@
 //   phi = sigma c1 / rho = 1 + kappa, psi = sigma^2 c2 / rho,
 //   A = phi / 2 - sigma^2 c2, B = psi / 2 - sigma^3 c3.
 // |w| <= eps makes a = O(eps), and kappa, A and w itself too.  So
-//   - x, r0^2, 1 / r0^3 (1 + kappa) and the sums of m x / r0^3 are FP64;
+//   - x, r0^2, 1 / r0^3 (1 + kappa) and the sums of m x / r0^3 (1 + kappa)
+//     are FP64;
 //   - kappa, and everything that multiplies w or is multiplied by A, is a
 //     double-word of about 2^-47 relative error, 2^-52 of the increment at
 //     eps = 2^-5.  Quantities near 1 or 1/2 are held as their small
@@ -37,12 +38,13 @@
 // Which pairs (weak_class): |w| <= 2^-5 r0 and mu <= 2^-10, the speeds
 // |t v_i|, |t v_j| below 2^-4 r0 (w is a difference of double-words, whose
 // error is relative to them), all factors well inside float's range; every
-// other pair takes the FP64 solve.  At that limit the measured error of the
-// velocity increment reaches the FP64 solve's (2.3 against 2.4 units of
-// 2^-53 r.m.s. between 2^-6 and 2^-5, 1.3 against 2.3 below 2^-8; of the
-// position increment 0.9 against 1.8 units of 2^-53 |t delta_v| / 2):
-// tests/test_weak_host.py.  A wider limit loses accuracy, a narrower one
-// sends more pairs to the FP64 solve (their number grows with the limit's
+// other pair takes the FP64 solve.  Up to that limit the velocity increments
+// are no less accurate than the map in plain FP64 arithmetic (units of 2^-53
+// r.m.s., here / plain FP64: 1.3 / 2.9 below 2^-9, 1.5 / 2.8 between 2^-7 and
+// 2^-6, 1.8 / 2.9 up to 2^-5.5, 2.2 / 2.9 up to 2^-5;
+// tests/test_weak_precision_host.py); the position's are off by 1.4 units of
+// 2^-53 |t delta_v| / 2 at most.  A wider limit loses accuracy, a narrower
+// one sends more pairs to the FP64 solve (their number grows with the limit's
 // inverse cube: 0.7 % of the pairs of a 1024-body Plummer sphere at step
 // 2^-8 with 2^-5, 5 % with 2^-6).
 #pragma once
@@ -182,8 +184,7 @@ DW_HD double dw_to_double(dw x)
 // Part of a pair's increments that do not depend on which particle takes
 // them: Q (FP64) multiplies the separation, K the small terms.
 struct WeakPair {
-    double Q;             // (1 + kappa - kl) / r0^3
-    float kl;             // the part of kappa below the last place of Q's FMA
+    double Q;             // (1 + kappa) / r0^3
     dw K, psi, Ap, Bp;    // 1 / r0^3, psi, A, B
 };
 
@@ -290,14 +291,17 @@ DW_HD void weak_solve(double r2, dw r2d, const dw xd[3], const dw w[3], dw M, We
     const dw ip = {ir, fmul(ir, rr)};
     const dw hp = fast_two_sum(0.5f, h2.h);
     const dw psi = dwu_norm(dwu_mul(dw{hp.h, fadd(hp.l, h2.l)}, ip));
-    // kappa' = (1 + kappa)(1 + 3e/2 + 15 e^2/8) - 1
+    // kappa' = (1 + kappa)(1 + 3e/2 + 15 e^2/8) - 1 as kp.h + kl', every
+    // product above 2^-54 in it, and both parts into the FP64 factor: the
+    // second one (up to 2^-28) as a term of the double-word sums instead, and
+    // without the products of second parts, made the error along x 3.1 units
+    // of 2^-53 r.m.s. where this is 2.3
     dw et = two_prod(1.5f, e.h);
-    et.l = fadd(ffma(1.5f, e.l, et.l), fmul(et.h, ffma(1.25f, ef, k1)));
-    dw kp = two_sum(k1, et.h);
-    kp.l = fadd(kp.l, fadd(kl, et.l));
+    et.l = ffma(1.5f, e.l, ffma(et.h, fmul(1.25f, ef), et.l));
+    const dw kp = two_sum(k1, et.h);
+    const float kq = ffma(et.h, k1, fadd(kl, ffma(et.h, kl, ffma(et.l, k1, et.l))));
     const double y3 = y2d * yd;
-    o.Q = fma(y3, widen(kp.h), y3);
-    o.kl = kp.l;
+    o.Q = fma(y3, widen(kp.h) + widen(fadd(kp.l, kq)), y3);
     o.K = K;
     o.psi = psi;
     o.Ap = dwu_norm(dwu_sub(dw{0.5f * k1, 0.5f * kl}, h2));
@@ -402,8 +406,7 @@ DW_HD void weak_add(const WeakParticle &a, const WeakParticle &b, const WeakDiff
     }
     const dw Kj = dwu_mul(b.mh, o.K), Ki = dwu_mul(a.mh, o.K);
     for (int q = 0; q < 3; ++q) {
-        dw e = dwu_mul(o.psi, d.w[q]);
-        e.l = ffma(o.kl, xd[q].h, e.l);
+        const dw e = dwu_mul(o.psi, d.w[q]);
         weak_acc(er[q], Kj, e);
         weak_acc(ec[q], Ki, e);
         const dw r = dwu_add(dwu_mul(o.Ap, xd[q]), dwu_mul(o.Bp, d.w[q]));
