@@ -47,6 +47,7 @@ struct Context {
     sakura_config cfg{};
     cudaStream_t stream = nullptr;
     unsigned *d_status = nullptr;
+    sakura::WeakChosen *d_choice = nullptr;  // the kernels of the run's weak steps
     unsigned long long *d_stats = nullptr;
     double *h_energy = nullptr;      // page-locked [3]: E, T, U
     double *h_energy_dev = nullptr;  // its address on the device
@@ -269,7 +270,7 @@ int step_device_mixed_grp(const double *src, double *dst, const double *masses, 
         g.timers.push_back(tm);
     }
     sakura::launch_apply_grp(dst, X, nullptr, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
-                             g.d_status, g.stream);
+                             g.d_status, {}, g.stream);
     rc = launch_error();
     if (rc) return rc;
     g.steps += 1;
@@ -393,6 +394,58 @@ sakura::WeakForm weak_kind()
                                                  : sakura::WeakForm::Guess;
 }
 
+// A weak step launches two sets of kernels, those of the weak pairs and those
+// that solve every pair; the prep kernel chooses one of them on the device
+// from a sample of the pairs, the other's return at once (StepGate).  The
+// lines lie where the two cost the same: 17 % strong pairs, 3 % in the
+// double-word form, whose solve of every pair is the cheaper one.  us per step
+// by the weak pairs' kernels / the others, Plummer spheres at multiples of the
+// step 2^-8 with (share of strong pairs): 2999 bodies FP64 seeded 4 x (1.9 %)
+// 259 / 768, 8 x (9.4 %) 456 / 775, 12 x (20 %) 828 / 785, 16 x (30 %) 1168 /
+// 793; double-word 2 x (0.3 %) 234 / 320, 4 x 282 / 320, 6 x (5 %) 381 / 321,
+// 16 x 1153 / 332; 8192 bodies 8 x 3245 / 5386, 12 x 6206 / 5439, double-word
+// 4 x 1656 / 2184, 6 x 2256 / 2189.
+constexpr int kStrongLimit = 174, kDf64StrongLimit = 31;  // of kWeakSample
+sakura::WeakChoice weak_choice(float *X3)
+{
+    const int limit = g.cfg.precision == SAKURA_PREC_DF64 ? kDf64StrongLimit : kStrongLimit;
+    return {g.d_choice, limit, g.cfg.precision == SAKURA_PREC_MIXED, X3};
+}
+
+// Tile launch shape of a grid, or of a kernel with bps blocks per SM: contiguous
+// tile-step ranges for W = 4 blocks <= T warps (step_common.cuh), Smax slots per tile.
+struct TileShape {
+    int64_t blocks, W, T;
+    int Smax;
+};
+TileShape tile_shape_of(int64_t n, int64_t blocks)
+{
+    const int64_t nb = (n + 31) / 32;
+    TileShape t;
+    t.T = nb * (nb + 1) / 2 * 32;
+    t.blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, t.T / 4));
+    t.W = t.blocks * 4;
+    t.Smax = (int)((32 * t.W + t.T - 1) / t.T + 1);
+    return t;
+}
+TileShape tile_shape(int64_t n, int bps)
+{
+    return tile_shape_of(n, g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks : (int64_t)g.sm_count * bps);
+}
+
+// Further arguments of the double-word form's kernels for every pair.
+sakura::DwArgs dw_args(const sakura::StepArgs &a, const float *X3)
+{
+    sakura::DwArgs da;
+    da.X3 = X3;
+    da.ptau32 = (float)(a.pre * a.tau);
+    da.t32 = (float)a.tau;
+    da.ptau = split_dw(a.pre * a.tau);
+    da.t = split_dw(a.tau);
+    da.qtau = split_dw(a.post * a.tau);
+    return da;
+}
+
 // The double-word form in row-group phases (step_df64.cu): prep (drift and
 // three-float copy), pair and apply kernels.
 int step_device_df64_grp(const double *src, double *dst, const double *masses, int64_t n,
@@ -431,13 +484,7 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
     a.guess = (g.cfg.guess == SAKURA_GUESS_TAYLOR || g.cfg.guess == SAKURA_GUESS_FP32) ? 2 : 0;
     a.status = g.d_status;
     a.stats = g.d_stats;
-    sakura::DwArgs da;
-    da.X3 = X3;
-    da.ptau32 = (float)(a.pre * dt);
-    da.t32 = (float)dt;
-    da.ptau = split_dw(a.pre * dt);
-    da.t = split_dw(dt);
-    da.qtau = split_dw(a.post * dt);
+    const sakura::DwArgs da = dw_args(a, X3);
     const bool timing = (g.cfg.flags & SAKURA_FLAG_TIMING) != 0;
     std::pair<cudaEvent_t, cudaEvent_t> tm{nullptr, nullptr};
     if (timing) {
@@ -451,7 +498,7 @@ int step_device_df64_grp(const double *src, double *dst, const double *masses, i
         g.timers.push_back(tm);
     }
     sakura::launch_apply_grp(dst, X, nullptr, nullptr, parts, n, L, blocks, post_drift, false, 0.0,
-                             g.d_status, g.stream);
+                             g.d_status, {}, g.stream);
     rc = launch_error();
     if (rc) return rc;
     g.steps += 1;
@@ -477,31 +524,47 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
     const bool learned = !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED &&
                          g.cfg.precision == SAKURA_PREC_FP64;
     const bool seed = g.cfg.guess == SAKURA_GUESS_FP32 && g.cfg.precision != SAKURA_PREC_DF64;
-    int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks
-                     : (int64_t)g.sm_count *
-                           (weak ? sakura::pair_step_grp_weak_blocks_per_sm(stats, weak_kind())
-                                 : sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed));
+    const bool df64 = g.cfg.precision == SAKURA_PREC_DF64;  // a weak step of that form
+    int64_t every_blocks = g.cfg.grid_blocks, blocks = g.cfg.grid_blocks;
+    if (every_blocks <= 0)
+        every_blocks = (int64_t)g.sm_count *
+                       (df64 ? sakura::pair_step_grp_df64_blocks_per_sm(stats)
+                             : sakura::pair_step_grp_blocks_per_sm(stats, learned, seed, mixed));
+    if (blocks <= 0)
+        blocks = weak ? (int64_t)g.sm_count *
+                            sakura::pair_step_grp_weak_blocks_per_sm(stats, weak_kind())
+                      : every_blocks;
     const sakura::GrpLayout L = sakura::make_grp_layout(n, sakura::kFp64GrpShape, blocks);
+    // the layout of the kernel that solves every pair
+    const sakura::GrpLayout Le = sakura::make_grp_layout(
+        n, df64 ? sakura::kDf64GrpShape : sakura::kFp64GrpShape, every_blocks);
     // scratch: X[7][n] doubles, row partials [Hmax][6][n], column partials
-    // [ng][6][n] and [blocks][6][32], then X32[10][n] floats (single-precision
-    // seed) and the weak pairs' rows [4][n] of 16 bytes
-    int rc = grow(g.partial, (size_t)(7 * n + (int64_t)(L.Hmax + L.ng) * 6 * n + blocks * 192 +
-                                      5 * n + (weak ? 8 * n + 1 : 0)) *
-                                 sizeof(double));
+    // [ng][6][n] and [blocks][6][32] (of either layout), then X32[10][n] floats
+    // (single-precision seed) or X3[20][n] (double-word form) and the weak
+    // pairs' rows [4][n] of 16 bytes
+    const int64_t sums = std::max((int64_t)(L.Hmax + L.ng) * 6 * n + blocks * 192,
+                                  (int64_t)(Le.Hmax + Le.ng) * 6 * n + every_blocks * 192);
+    const int64_t head = 7 * n + sums + (df64 ? 10 * n : 5 * n);
+    int rc = grow(g.partial, (size_t)(head + (weak ? 8 * n + 1 : 0)) * sizeof(double));
     if (rc) return rc;
     double *X = (double *)g.partial.ptr;
-    sakura::GrpParts parts;
-    parts.row = X + 7 * n;
-    parts.col = parts.row + (int64_t)L.Hmax * 6 * n;
-    parts.colx = parts.col + (int64_t)L.ng * 6 * n;
-    float *X32 = (seed || mixed) ? (float *)(parts.colx + blocks * 192) : nullptr;
+    auto parts_of = [&](const sakura::GrpLayout &l) {
+        sakura::GrpParts p;
+        p.row = X + 7 * n;
+        p.col = p.row + (int64_t)l.Hmax * 6 * n;
+        p.colx = p.col + (int64_t)l.ng * 6 * n;
+        return p;
+    };
+    const sakura::GrpParts parts = parts_of(L);
+    float *floats = (float *)(X + 7 * n + sums);
+    float *X32 = (seed || mixed) ? floats : nullptr, *X3 = df64 ? floats : nullptr;
     // the weak rows, 16-byte aligned
-    const int64_t head = 12 * n + (int64_t)(L.Hmax + L.ng) * 6 * n + blocks * 192;
     float4 *rows = weak ? (float4 *)(X + head + (head & 1)) : nullptr;
     const double drift = order == 2 ? 0.5 * dt : (order == 1 ? 0.0 : dt);
     const double post_drift = order == 2 ? 0.5 * dt : (order == 1 ? dt : 0.0);
     if (!prepped && weak)
-        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, g.stream);
+        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, weak_choice(X3),
+                                 g.stream);
     else if (!prepped)
         sakura::launch_prep_step(src, masses, X, X32, n, drift, g.d_status, g.stream);
     sakura::StepArgs a;
@@ -532,10 +595,19 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
         tm = take_timer();
         cudaEventRecord(tm.first, g.stream);
     }
+    sakura::GrpAlt alt = {};
     if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
+        a.gate = {&g.d_choice->every, 0};
         sakura::launch_pair_step_grp_weak(a, ws, L, parts, (int)blocks, stats, weak_kind(),
                                           g.stream);
+        alt = {&g.d_choice->every, parts_of(Le), Le, every_blocks, X3};
+        a.gate.open = 1;
+        if (df64)
+            sakura::launch_pair_step_grp_df64(a, dw_args(a, X3), Le, alt.parts, (int)every_blocks,
+                                              stats, g.stream);
+        else
+            sakura::launch_pair_step_grp(a, Le, alt.parts, (int)every_blocks, stats, g.stream);
     } else {
         sakura::launch_pair_step_grp(a, L, parts, (int)blocks, stats, g.stream);
     }
@@ -545,7 +617,7 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
         g.timers.push_back(tm);
     }
     sakura::launch_apply_grp(dst, X, X32, rows, parts, n, L, blocks, post_drift, fuse, next_drift,
-                             g.d_status, g.stream);
+                             g.d_status, alt, g.stream);
     rc = launch_error();
     if (rc) return rc;
     g.steps += 1;
@@ -589,44 +661,43 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
     const bool learned = !df64 && !dwf && !mixed && g.cfg.guess == SAKURA_GUESS_LEARNED;
     const bool seed = !df64 && !dwf && g.cfg.guess == SAKURA_GUESS_FP32;
     const int64_t nb = (n + 31) / 32;
-    const int64_t tiles = nb * (nb + 1) / 2;
-    const int bps = df64   ? sakura::pair_step_df64_blocks_per_sm(stats)
-                    : weak ? sakura::pair_step_weak_blocks_per_sm(stats, weak_kind())
-                           : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
-    // contiguous tile-step ranges for W <= T warps (step_common.cuh)
-    const int64_t T = tiles * 32;
-    int64_t blocks = g.cfg.grid_blocks > 0 ? g.cfg.grid_blocks : (int64_t)g.sm_count * bps;
-    blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, T / 4));
+    const int every_bps = df64 || dwf
+                              ? sakura::pair_step_df64_blocks_per_sm(stats)
+                              : sakura::pair_step_sym_blocks_per_sm(stats, learned, seed, mixed);
+    TileShape shape =
+        tile_shape(n, weak ? sakura::pair_step_weak_blocks_per_sm(stats, weak_kind()) : every_bps);
+    const TileShape every = tile_shape(n, every_bps);  // the kernel that solves every pair
+    const int64_t T = shape.T;
     // mixed form: two tile-steps per warp where one would take more than one
     // block per SM and two take at most two (256 bodies, four steps: 89 us
     // against 107; 333: 108 against 126; outside that range one is faster:
     // 128 bodies 80 against 89)
     if (mixed && !weak && g.cfg.grid_blocks <= 0 && T / 4 > g.sm_count &&
         T / 8 <= 2 * (int64_t)g.sm_count)
-        blocks = T / 8;
-    const int64_t W = blocks * 4;
-    const int Smax = (int)((32 * W + T - 1) / T + 1);
-    const int64_t nslots = nb * Smax;
+        shape = tile_shape_of(n, T / 8);
+    const int64_t blocks = shape.blocks, W = shape.W;
+    const int Smax = shape.Smax;
+    const int64_t nslots = nb * (weak ? std::max(Smax, every.Smax) : Smax);
     // scratch: X[7][n] doubles, tile partials [nslots][6][n] (doubles, or
-    // double-words of two floats), then (df64) X3[20][n] or (seed) X32[10][n]
-    // floats and the weak pairs' rows [4][n] of 16 bytes
-    int rc = grow(g.partial, (size_t)(7 * n + nslots * 6 * n + (df64 ? 10 * n : 5 * n) +
-                                      (weak ? 8 * n + 1 : 0)) *
-                                 sizeof(double));
+    // double-words of two floats), then (double-word form) X3[20][n] or (seed)
+    // X32[10][n] floats and the weak pairs' rows [4][n] of 16 bytes
+    const int64_t head = 7 * n + nslots * 6 * n + (df64 || dwf ? 10 * n : 5 * n);
+    int rc = grow(g.partial, (size_t)(head + (weak ? 8 * n + 1 : 0)) * sizeof(double));
     if (rc) return rc;
     double *X = (double *)g.partial.ptr;
     double *partial = X + 7 * n;
-    float *X3 = (float *)(partial + nslots * 6 * n);
-    float *X32 = (seed || mixed) ? X3 : nullptr;
+    float *floats = (float *)(partial + nslots * 6 * n);
+    float *X3 = df64 || dwf ? floats : nullptr;
+    float *X32 = (seed || mixed) ? floats : nullptr;
     // the weak rows, 16-byte aligned
-    const int64_t head = 12 * n + nslots * 6 * n;
     float4 *rows = weak ? (float4 *)(X + head + (head & 1)) : nullptr;
     const double drift = order == 2 ? 0.5 * dt : (order == 1 ? 0.0 : dt);
     const double post_drift = order == 2 ? 0.5 * dt : (order == 1 ? dt : 0.0);
     if (df64)
         sakura::launch_prep_df64(src, masses, X, X3, n, drift, g.d_status, g.stream);
     else if (!prepped && weak)
-        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, g.stream);
+        sakura::launch_prep_weak(src, masses, X, X32, rows, n, dt, g.d_status, weak_choice(X3),
+                                 g.stream);
     else if (!prepped)
         sakura::launch_prep_step(src, masses, X, X32, n, drift, g.d_status, g.stream);
     sakura::StepArgs a;
@@ -659,18 +730,17 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         cudaEventRecord(tm.first, g.stream);
     }
     if (df64) {
-        sakura::DwArgs da;
-        da.X3 = X3;
-        da.ptau32 = (float)(a.pre * dt);
-        da.t32 = (float)dt;
-        da.ptau = split_dw(a.pre * dt);
-        da.t = split_dw(dt);
-        da.qtau = split_dw(a.post * dt);
-        sakura::launch_pair_step_df64(a, da, Smax, T, (int)blocks, stats, g.stream);
+        sakura::launch_pair_step_df64(a, dw_args(a, X3), Smax, T, (int)blocks, stats, g.stream);
     } else if (weak) {
         const sakura::WeakStep ws{rows, 1.0 / dt};
-        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, weak_kind(),
-                                          g.stream);
+        a.gate = {&g.d_choice->every, 0};
+        sakura::launch_pair_step_weak(a, ws, Smax, T, (int)blocks, stats, weak_kind(), g.stream);
+        a.gate.open = 1;
+        if (dwf)
+            sakura::launch_pair_step_df64(a, dw_args(a, X3), every.Smax, T, (int)every.blocks,
+                                          stats, g.stream);
+        else
+            sakura::launch_pair_step_sym(a, every.Smax, T, (int)every.blocks, stats, g.stream);
     } else {
         sakura::launch_pair_step_sym(a, Smax, T, (int)blocks, stats, g.stream);
     }
@@ -682,8 +752,10 @@ int step_device_sym(const double *src, double *dst, const double *masses, int64_
         sakura::launch_apply_df64(dst, X, partial, n, Smax, W, T, post_drift, g.d_status,
                                   g.stream);
     else
-        sakura::launch_apply_sym(dst, X, X32, rows, partial, n, Smax, W, T, post_drift,
-                                 fuse, next_drift, g.d_status, g.stream);
+        sakura::launch_apply_sym(
+            dst, X, X32, rows, partial, n, Smax, W, T, post_drift, fuse, next_drift, g.d_status,
+            weak ? sakura::SymAlt{&g.d_choice->every, every.Smax, every.W, X3} : sakura::SymAlt{},
+            g.stream);
     rc = launch_error();
     if (rc) return rc;
     g.steps += 1;
@@ -937,7 +1009,8 @@ const double *step_masses(int64_t n) { return (const double *)g.partial.ptr + 6 
 // reallocated in between: every sub-step of a run has the same n, options and
 // weak, on which alone its size depends.  Where fusable, every apply kernel
 // but the last also drifts for the next sub-step, so only the first sub-step
-// runs a prep kernel (the same arithmetic: results are unchanged).
+// runs a prep kernel (the same arithmetic: results are unchanged); where it
+// chooses between two sets of kernels (weak_choice), it does so for the run.
 int run_substeps(const double *src, double *mid, double *dst, const double *masses, int64_t n,
                  double dt, int order, int nsteps)
 {
@@ -1111,6 +1184,8 @@ int sakura_init(const sakura_config *cfg)
     if (g.init && g.cfg.device != c.device) sakura_finalize();
     if (!g.init) {
         if (cudaMalloc(&g.d_status, sizeof(unsigned)) != cudaSuccess) return SAKURA_E_NOMEM;
+        if (cudaMalloc(&g.d_choice, sizeof(*g.d_choice)) != cudaSuccess) return SAKURA_E_NOMEM;
+        if (cudaMemset(g.d_choice, 0, sizeof(*g.d_choice)) != cudaSuccess) return SAKURA_E_CUDA;
         if (cudaMalloc(&g.d_stats, sakura::kStatCount * sizeof(unsigned long long)) !=
             cudaSuccess)
             return SAKURA_E_NOMEM;
@@ -1153,6 +1228,7 @@ int sakura_finalize(void)
         b->bytes = 0;
     }
     cudaFree(g.d_status);
+    cudaFree(g.d_choice);
     cudaFree(g.d_stats);
     if (g.h_energy) cudaFreeHost(g.h_energy);
     if (g.h_status) cudaFreeHost(g.h_status);

@@ -49,6 +49,19 @@ constexpr int kStatFp32Pairs = 4;
 constexpr int kStatCarries = 5;
 constexpr int kStatCount = 8;
 
+// A kernel that runs where *p == open and returns at once elsewhere (p null:
+// it runs): of the kernels that a step launches for its weak pairs and for
+// every pair, those that the prep kernel chose on the device (step_weak.cu).
+struct StepGate {
+    const int *p;
+    int open;
+};
+
+__device__ __forceinline__ bool gate_closed(const StepGate &g)
+{
+    return g.p && __ldcg(g.p) != g.open;
+}
+
 struct StepArgs {
     const double *X;      // [7][n] drifted positions, velocities, masses (prep kernel)
     double *partial;      // [slots][6][n] row sums of mu_ij delta / m_i, split by warp
@@ -71,6 +84,7 @@ struct StepArgs {
     int mixed;
     ClassRule rule;
     float post32;
+    StepGate gate;
 };
 
 // extra arguments of the mixed-precision pair kernel
@@ -163,10 +177,19 @@ void launch_pair_step_sym(const StepArgs &a, int Smax, int64_t T, int blocks, bo
                           cudaStream_t s);
 // fuse: also apply the next sub-step's drift next_drift and write its
 // drifted copy to X (and X32, if not null), replacing the next prep kernel
+// alt: the partial sums' shape where *alt.p != 0 (alt.p null: Smax and W
+// always).  X3 not null: the sums are then double-words, and with fuse the
+// three-float copy X3[20][n] of the drifted state is written too
+struct SymAlt {
+    const int *p;
+    int Smax;
+    int64_t W;
+    float *X3;
+};
 void launch_apply_sym(double *state, double *X, float *X32, float4 *rows,
                       const double *partial, int64_t n,
                       int Smax, int64_t W, int64_t T, double post_drift, bool fuse,
-                      double next_drift, unsigned *status, cudaStream_t s);
+                      double next_drift, unsigned *status, const SymAlt &alt, cudaStream_t s);
 
 // number of partial-sum slots per row for W warps
 int pair_step_slots(int64_t n, int64_t W);

@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(128)
 {
     __shared__ int queue[4][64];
     __shared__ float2 qres[4][32][12];  // queued results as double-words
-    griddep_wait();    // X and X3 from the prep kernel
+    griddep_wait();  // X and X3 from the prep kernel
+    if (gate_closed(a.gate)) return;
     griddep_launch();  // the apply kernel may begin launching
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -376,7 +377,8 @@ __global__ void __launch_bounds__(kDf64GrpWarps * 32, 1)
         reinterpret_cast<int(*)[64]>(gsm + sizeof(float4) * (G * 3 + 2 * 5) * WIN * 32);
     int(*queue_j)[64] = queue_i + G;
     float2(*qres)[32][12] = reinterpret_cast<float2(*)[32][12]>(queue_j + G);
-    griddep_wait();    // X and X3 from the prep kernel
+    griddep_wait();  // X and X3 from the prep kernel
+    if (gate_closed(a.gate)) return;
     griddep_launch();  // the apply kernel may begin launching
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;

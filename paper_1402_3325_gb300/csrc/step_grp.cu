@@ -87,10 +87,15 @@ constexpr int kGrpApplyWarps = 8;
 __global__ void __launch_bounds__(32 * kGrpApplyWarps)
     apply_grp_kernel(double *state, double *X, float *X32, float4 *rows, GrpParts parts,
                      int64_t n, GrpLayout L, int64_t B, double post_drift, int fuse, double next_drift,
-                     unsigned *status)
+                     unsigned *status, GrpAlt alt)
 {
     __shared__ double red[kGrpApplyWarps][2][32];
     griddep_wait();  // the pair kernel's partials
+    if (alt.p && __ldcg(alt.p)) {
+        parts = alt.parts;
+        L = alt.L;
+        B = alt.blocks;
+    }
     // Without fuse, a kernel that follows reads this one's output only after
     // its own griddep_wait or is launched plainly, so it may begin launching
     // now.  With fuse the next kernel is a persistent pair kernel whose
@@ -164,6 +169,7 @@ __global__ void __launch_bounds__(32 * kGrpApplyWarps)
             X32[(3 + q) * n + ip] = __double2float_rn(x - (double)hi);
             X32[(6 + q) * n + ip] = __double2float_rn(v1);
         }
+        if (alt.X3) tf_row_component(alt.X3, n, ip, q, x, v1);
         if (rows) {
             const double tau = 2.0 * next_drift;
             weak_row_component(rows, n, ip, q, x1n, v1, tau);
@@ -174,7 +180,7 @@ __global__ void __launch_bounds__(32 * kGrpApplyWarps)
 
 void launch_apply_grp(double *state, double *X, float *X32, float4 *rows, const GrpParts &parts,
                       int64_t n, const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
-                      double next_drift, unsigned *status, cudaStream_t s)
+                      double next_drift, unsigned *status, const GrpAlt &alt, cudaStream_t s)
 {
     GrpParts pv = parts;
     GrpLayout Lv = L;
@@ -182,7 +188,7 @@ void launch_apply_grp(double *state, double *X, float *X32, float4 *rows, const 
     int f = fuse ? 1 : 0;
     void *args[] = {(void *)&state,      (void *)&X, (void *)&X32, (void *)&rows, (void *)&pv,
                     (void *)&n,          (void *)&Lv, (void *)&B,         (void *)&post_drift,
-                    (void *)&f,          (void *)&next_drift, (void *)&status};
+                    (void *)&f,          (void *)&next_drift, (void *)&status, (void *)&alt};
     launch_pdl((const void *)apply_grp_kernel, dim3((unsigned)((n + 31) / 32), 3),
                dim3(32 * kGrpApplyWarps), args, 0, s);
 }
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32,
     __nv_bfloat16 *mlpStage =
         reinterpret_cast<__nv_bfloat16 *>(gsm + grp_base_smem(WIN, F32) + sizeof(MlpWeights));
     griddep_wait();    // X (and X32) from the prep kernel or the previous apply kernel
+    if (gate_closed(a.gate)) return;
     griddep_launch();  // the apply kernel may begin launching
     if (LEARNED) mlp_load_shared(*mlpW, a.mlp);
     const int lane = threadIdx.x & 31;

@@ -22,10 +22,17 @@ int pair_step_grp_mixed_blocks_per_sm(bool stats, bool seed);
 // Eqs. 27b-d for the row-group layout; fuse: also the next sub-step's drift
 // (next_drift), writing its drifted copy to X (and X32, if not null) as the
 // prep kernel would, so that a run of steps needs no prep kernel after its
-// first
+// first; alt as for launch_apply_sym, but the sums always in FP64
+struct GrpAlt {
+    const int *p;
+    GrpParts parts;
+    GrpLayout L;
+    int64_t blocks;
+    float *X3;
+};
 void launch_apply_grp(double *state, double *X, float *X32, float4 *rows, const GrpParts &parts,
                       int64_t n, const GrpLayout &L, int64_t blocks, double post_drift, bool fuse,
-                      double next_drift, unsigned *status, cudaStream_t s);
+                      double next_drift, unsigned *status, const GrpAlt &alt, cudaStream_t s);
 // the symmetric FP64 pair kernel in row-group phases (a.mlp: learned guess;
 // a.X32: single-precision seed; a.mixed: the mixed form's inline class test,
 // a.mixed == 2 with the seed, as in launch_pair_step_sym)

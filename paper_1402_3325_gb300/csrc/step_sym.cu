@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(128, MIXED ? 2 : ((SEED || LEARNED) ? 3 : 4))
     extern __shared__ __align__(16) unsigned char dsm[];
     MlpWeights *mlpW = reinterpret_cast<MlpWeights *>(dsm);
     __nv_bfloat16 *mlpStage = reinterpret_cast<__nv_bfloat16 *>(dsm + sizeof(MlpWeights));
-    griddep_wait();    // X from the prep kernel
+    griddep_wait();  // X from the prep kernel
+    if (gate_closed(a.gate)) return;
     griddep_launch();  // the apply kernel may begin launching
     if (LEARNED) mlp_load_shared(*mlpW, a.mlp);
     const int lane = threadIdx.x & 31;
@@ -261,13 +262,24 @@ __global__ void __launch_bounds__(128, MIXED ? 2 : ((SEED || LEARNED) ? 3 : 4))
 // first; the next pair kernel may then begin launching at once.
 constexpr int kApplyWarps = 16;
 
+// the double-word of two floats in the bits of x
+__device__ __forceinline__ double words_sum(double x)
+{
+    return f2d(__int_as_float(__double2loint(x))) + f2d(__int_as_float(__double2hiint(x)));
+}
+
 __global__ void __launch_bounds__(32 * kApplyWarps)
     apply_sym_kernel(double *state, double *X, float *X32, float4 *rows, const double *partial,
                      int64_t n, int Smax, int64_t W, int64_t T, double post_drift, int fuse,
-                     double next_drift, unsigned *status)
+                     double next_drift, unsigned *status, SymAlt alt)
 {
     __shared__ double red[kApplyWarps][2][32];
     griddep_wait();  // the pair kernel's partials
+    const bool every = alt.p && __ldcg(alt.p), words = every && alt.X3;
+    if (every) {
+        Smax = alt.Smax;
+        W = alt.W;
+    }
     // Without fuse, a kernel that follows reads this one's output only after
     // its own griddep_wait or is launched plainly, so it may begin launching
     // now.  With fuse the next kernel is a persistent pair kernel whose
@@ -293,8 +305,13 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
             const int segs = sym_segments(tile, W, T);
             for (int o = 0; o < segs; ++o) {
                 const int64_t k = Q * Smax + o;
-                er[u] += partial[(k * 6 + q) * n + i];
-                ev[u] += partial[(k * 6 + 3 + q) * n + i];
+                double r = partial[(k * 6 + q) * n + i], v = partial[(k * 6 + 3 + q) * n + i];
+                if (words) {
+                    r = words_sum(r);
+                    v = words_sum(v);
+                }
+                er[u] += r;
+                ev[u] += v;
                 u ^= 1;
             }
         }
@@ -325,6 +342,7 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
             X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
             X32[(6 + q) * n + i] = __double2float_rn(v1);
         }
+        if (alt.X3) tf_row_component(alt.X3, n, i, q, x, v1);
         if (rows) {
             const double tau = 2.0 * next_drift;
             weak_row_component(rows, n, i, q, x1, v1, tau);
@@ -390,12 +408,13 @@ void launch_pair_step_sym(const StepArgs &a, int Smax, int64_t T, int blocks, bo
 
 void launch_apply_sym(double *state, double *X, float *X32, float4 *rows, const double *partial,
                       int64_t n, int Smax, int64_t W, int64_t T, double post_drift, bool fuse,
-                      double next_drift, unsigned *status, cudaStream_t s)
+                      double next_drift, unsigned *status, const SymAlt &alt, cudaStream_t s)
 {
     int f = fuse ? 1 : 0;
     void *args[] = {(void *)&state,      (void *)&X, (void *)&X32, (void *)&rows, (void *)&partial,
                     (void *)&n,          (void *)&Smax, (void *)&W, (void *)&T,
-                    (void *)&post_drift, (void *)&f, (void *)&next_drift, (void *)&status};
+                    (void *)&post_drift, (void *)&f, (void *)&next_drift, (void *)&status,
+                    (void *)&alt};
     launch_pdl((const void *)apply_sym_kernel, dim3((unsigned)((n + 31) / 32), 3),
                dim3(32 * kApplyWarps), args, 0, s);
 }

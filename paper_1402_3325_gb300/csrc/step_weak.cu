@@ -10,7 +10,13 @@
 // warp's queue in shared memory and are solved 32 at a time by the seeded
 // FP64 solver, so that a rare close pair does not make its warp run a
 // 75-instruction FP64 solve for one lane; a step with more than
-// kWeakInline strong lanes solves them at once.
+// kWeakInline strong lanes solves them at once.  Steps whose pairs are strong
+// in larger part than that pays for take the kernels that solve every pair
+// (step_sym.cu, step_grp.cu, step_df64.cu): both are launched, and the prep
+// kernel's choice (sample_classes) lets one of them return at once, 1 us per
+// step.  Separations out of the class's range, us per step with this kernel
+// alone -> so: 8192 bodies FP64 8000 -> 5220, double-word 6680 -> 2230; 2999
+// bodies 1105 -> 766, double-word 949 -> 351.
 //
 // Bound: the FP64 pipe (16 FP64 instructions per pair and 16 cycles each)
 // and the issue slots (950 instructions per pair and warp) nearly alike: ncu
@@ -36,8 +42,10 @@
 
 namespace sakura {
 
-// Strong lanes of a step that are queued at most: a batch solve of more than
-// 8 lanes in place costs no more than a quarter of one in the queue.
+// Strong lanes of a step that are queued at most.  Solved in place, more lanes
+// than these take a batch for themselves, at most 32 / 9 times what they take
+// in the queue; steps with as many are rare in the runs that take this kernel
+// (prep_weak_kernel chooses the others where one pair in six is strong).
 constexpr int kWeakInline = 8;
 // entries of a warp's queue on tiles: a segment's, and a rest below one batch
 constexpr int kWeakQueue = 32 * kWeakInline + 31;
@@ -370,6 +378,7 @@ __global__ void __launch_bounds__(128, 3)
     __shared__ double res[128][12];
     __shared__ int cnt[4];
     griddep_wait();
+    if (gate_closed(a.gate)) return;
     griddep_launch();
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -485,6 +494,7 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
         reinterpret_cast<int2(*)[32 * kWeakInline * WIN]>(res + 32 * G);
     __shared__ int cnt[G];
     griddep_wait();
+    if (gate_closed(a.gate)) return;
     griddep_launch();
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -607,13 +617,65 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
     s.finish<STATS>(a, lane);
 }
 
+// Which kernels a run's steps take: those of the weak pairs, or, where more
+// than limit of kWeakSample pairs of the state before the run are strong
+// (under the mixed form's rule: or not certainly unbound), those that solve
+// every pair.  The pairs are drawn by a hash of their number, so the choice
+// depends on the state alone.  A pair per thread in 16 blocks: the test's 40
+// FP64 instructions take 10 us when one block makes them all.
+constexpr int kPrepThreads = 64, kSampleBlocks = kWeakSample / kPrepThreads;
+
+__device__ __forceinline__ WeakParticle sample_particle(const double *state, const double *mass,
+                                                        int64_t n, int64_t i, double tau)
+{
+    WeakParticle p;
+    p.x = state[i];
+    p.y = state[n + i];
+    p.z = state[2 * n + i];
+    p.mt = tau * mass[i];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) p.w[q] = {(float)(tau * state[(3 + q) * n + i]), 0.0f};
+    p.mh = {(float)(tau * p.mt), 0.0f};
+    return p;
+}
+
+__device__ __forceinline__ void sample_classes(const double *state, const double *mass, int64_t n,
+                                               double tau, int block, const WeakChoice &ch)
+{
+    uint32_t h = (uint32_t)(kPrepThreads * block + threadIdx.x + 1) * 0x9e3779b1u;
+    h = (h ^ (h >> 15)) * 0x85ebca77u;
+    h ^= h >> 13;
+    const uint32_t g = (h * 0xc2b2ae3du) ^ (h >> 16);
+    const int64_t i = (int64_t)(((uint64_t)h * (uint64_t)n) >> 32);
+    int64_t j = i + 1 + (int64_t)(((uint64_t)g * (uint64_t)(n - 1)) >> 32);
+    if (j >= n) j -= n;
+    const WeakParticle a = sample_particle(state, mass, n, i, tau);
+    const WeakParticle b = sample_particle(state, mass, n, j, tau);
+    const float sa = weak_speed2(a);
+    WeakDiff d;
+    const bool weak = weak_class(a, sa, b, d) && (!ch.unbound || weak_unbound(a, sa, b, d));
+    const unsigned strong = __syncthreads_count(!weak);
+    if (threadIdx.x != 0) return;
+    // the counts' sum and, above it, their number; the last block leaves zero
+    const unsigned before = atomicAdd(&ch.p->sum, strong + (1u << 16));
+    if (before >> 16 != kSampleBlocks - 1) return;
+    ch.p->sum = 0u;
+    ch.p->every = (before & 0xffffu) + strong > (unsigned)ch.limit ? 1 : 0;
+}
+
 // Eq. 27a (order 2), the drifted state with its float copy for the FP64
-// solves, and the rows of the weak pairs; one thread per particle
+// solves, and the rows of the weak pairs; one thread per particle, and the
+// first kSampleBlocks blocks for the choice of the kernels
 __global__ void prep_weak_kernel(const double *state, const double *mass, double *X, float *X32,
-                                 float4 *rows, int64_t n, double tau, unsigned *status)
+                                 float4 *rows, int64_t n, double tau, unsigned *status,
+                                 WeakChoice ch)
 {
     griddep_launch();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x < kSampleBlocks) {
+        sample_classes(state, mass, n, tau, blockIdx.x, ch);
+        return;
+    }
+    const int64_t i = (int64_t)(blockIdx.x - kSampleBlocks) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double m = mass[i], drift = 0.5 * tau;
     if (!(m > 0.0)) atomicOr(status, kStatusMass);
@@ -629,9 +691,11 @@ __global__ void prep_weak_kernel(const double *state, const double *mass, double
             X32[(3 + q) * n + i] = __double2float_rn(x - (double)hi);
             X32[(6 + q) * n + i] = __double2float_rn(v);
         }
+        if (ch.X3) tf_row_component(ch.X3, n, i, q, x, v);
         weak_row_component(rows, n, i, q, x0, v, tau);
     }
     X[6 * n + i] = m;
+    if (ch.X3) tf_row_mass(ch.X3, n, i, m);
     if (X32) X32[9 * n + i] = __double2float_rn(m);
     weak_row_mass(rows, n, i, m, tau);
 }
@@ -959,11 +1023,12 @@ void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpL
 }
 
 void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
-                      float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s)
+                      float4 *rows, int64_t n, double tau, unsigned *status,
+                      const WeakChoice &ch, cudaStream_t s)
 {
-    const int threads = 64;
-    prep_weak_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
-        state, mass, X, X32, rows, n, tau, status);
+    const int threads = kPrepThreads;
+    prep_weak_kernel<<<kSampleBlocks + (unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
+        state, mass, X, X32, rows, n, tau, status, ch);
 }
 
 }  // namespace sakura

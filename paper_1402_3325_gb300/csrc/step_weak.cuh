@@ -20,8 +20,25 @@ struct WeakStep {
 // guess (no X32, no statistics).
 enum class WeakForm { Fp64, Df64, Mixed, Guess, Learned };
 
+// The choice of a run's kernels, by the prep kernel from sampled pairs of the
+// state: p->every = 0 those of the weak pairs, 1 those that solve every pair
+// (more than limit of kWeakSample pairs strong; unbound: weak pairs are
+// unbound ones only, the mixed form's rule).
+constexpr int kWeakSample = 1024;
+struct WeakChosen {
+    int every;
+    unsigned sum;  // of the sample's blocks; zero between runs
+};
+struct WeakChoice {
+    WeakChosen *p;
+    int limit;
+    bool unbound;
+    float *X3;  // three-float copy that the prep kernel writes (double-word form) or null
+};
+
 void launch_prep_weak(const double *state, const double *mass, double *X, float *X32,
-                      float4 *rows, int64_t n, double tau, unsigned *status, cudaStream_t s);
+                      float4 *rows, int64_t n, double tau, unsigned *status, const WeakChoice &ch,
+                      cudaStream_t s);
 void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t T, int blocks,
                            bool stats, WeakForm form, cudaStream_t s);
 int pair_step_weak_blocks_per_sm(bool stats, WeakForm form);

@@ -27,9 +27,10 @@ bool state_ok(const double *src, const double *mass, const double *X, int64_t n)
 }  // namespace
 
 void launch_prep_weak(const double *src, const double *mass, double *X, float *X32, float4 *rows,
-                      int64_t n, double, unsigned *, cudaStream_t)
+                      int64_t n, double, unsigned *, const WeakChoice &ch, cudaStream_t)
 {
-    note("prep_weak", state_ok(src, mass, X, n) && (size_t)rows % 16 == 0 &&
+    note("prep_weak", held(ch.p, sizeof(*ch.p)) &&
+                          (!ch.X3 || held(ch.X3, 80 * (size_t)n)) && state_ok(src, mass, X, n) && (size_t)rows % 16 == 0 &&
                           held(rows, 64 * (size_t)n) && (!X32 || held(X32, 40 * (size_t)n)));
     std::memcpy(X + 6 * n, mass, doubles(n));
 }
@@ -59,19 +60,34 @@ void launch_copy_state(const double *src, const double *mass, double *dst, doubl
 namespace {
 bool args_ok(const StepArgs &a)
 {
-    return held(a.X, doubles(7 * a.n)) && (!a.X32 || held(a.X32, 40 * (size_t)a.n));
+    return held(a.X, doubles(7 * a.n)) && (!a.X32 || held(a.X32, 40 * (size_t)a.n)) &&
+           (!a.gate.p || held(a.gate.p, sizeof(int)));
+}
+
+// a weak step's other set of kernels, which solves every pair: "every_..."
+void note_pairs(const char *name, const StepArgs &a, bool ok)
+{
+    static char every[32];
+    std::strcat(std::strcpy(every, "every_"), name);
+    note(a.gate.p && a.gate.open == 1 ? every : name, ok);
+}
+
+// the tiles' partial sums
+bool slots_ok(const StepArgs &a, int Smax)
+{
+    return held(a.partial, doubles((a.n + 31) / 32 * Smax * 6 * a.n));
 }
 }  // namespace
 
-void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int, int64_t, int, bool, WeakForm,
-                           cudaStream_t)
+void launch_pair_step_weak(const StepArgs &a, const WeakStep &ws, int Smax, int64_t, int, bool,
+                           WeakForm, cudaStream_t)
 {
-    note("weak", args_ok(a) && held(ws.rows, 64 * (size_t)a.n));
+    note("weak", args_ok(a) && slots_ok(a, Smax) && a.gate.p && held(ws.rows, 64 * (size_t)a.n));
 }
 void launch_pair_step_grp_weak(const StepArgs &a, const WeakStep &ws, const GrpLayout &,
                                const GrpParts &parts, int blocks, bool, WeakForm, cudaStream_t)
 {
-    note("grp_weak", args_ok(a) && held(ws.rows, 64 * (size_t)a.n) &&
+    note("grp_weak", args_ok(a) && a.gate.p && held(ws.rows, 64 * (size_t)a.n) &&
                          held(parts.colx, doubles(192 * (int64_t)blocks)));
 }
 void launch_pair_step_weak_small(const StepArgs &a, const WeakSmall &ws, int, bool, bool, WeakForm,
@@ -86,14 +102,14 @@ void launch_apply_weak_small(const double *src, double *dst, const double *, int
 {
     note("small_apply", held(src, doubles(6 * n)) && held(dst, doubles(6 * n)));
 }
-void launch_pair_step_sym(const StepArgs &a, int, int64_t, int, bool, cudaStream_t)
+void launch_pair_step_sym(const StepArgs &a, int Smax, int64_t, int, bool, cudaStream_t)
 {
-    note("sym", args_ok(a));
+    note_pairs("sym", a, args_ok(a) && slots_ok(a, Smax));
 }
-void launch_pair_step_df64(const StepArgs &a, const DwArgs &da, int, int64_t, int, bool,
+void launch_pair_step_df64(const StepArgs &a, const DwArgs &da, int Smax, int64_t, int, bool,
                            cudaStream_t)
 {
-    note("df64", args_ok(a) && held(da.X3, 80 * (size_t)a.n));
+    note_pairs("df64", a, args_ok(a) && slots_ok(a, Smax) && held(da.X3, 80 * (size_t)a.n));
 }
 void launch_pair_step_fp64(const StepArgs &a, int, int, bool, cudaStream_t)
 {
@@ -103,31 +119,34 @@ void launch_pair_step_mixed(const StepArgs &a, const MixedArgs &, int, bool, cud
 {
     note("ordered_mixed", args_ok(a));
 }
-void launch_pair_step_grp(const StepArgs &a, const GrpLayout &, const GrpParts &, int, bool,
-                          cudaStream_t)
+void launch_pair_step_grp(const StepArgs &a, const GrpLayout &, const GrpParts &parts, int blocks,
+                          bool, cudaStream_t)
 {
-    note("grp", args_ok(a));
+    note_pairs("grp", a, args_ok(a) && held(parts.colx, doubles(192 * (int64_t)blocks)));
 }
 void launch_pair_step_grp_mixed(const StepArgs &a, const MixedArgs &, const GrpLayout &,
                                 const GrpParts &, int, bool, cudaStream_t)
 {
     note("grp_mixed", args_ok(a));
 }
-void launch_pair_step_grp_df64(const StepArgs &a, const DwArgs &, const GrpLayout &,
-                               const GrpParts &, int, bool, cudaStream_t)
+void launch_pair_step_grp_df64(const StepArgs &a, const DwArgs &da, const GrpLayout &,
+                               const GrpParts &parts, int blocks, bool, cudaStream_t)
 {
-    note("grp_df64", args_ok(a));
+    note_pairs("grp_df64", a, args_ok(a) && held(da.X3, 80 * (size_t)a.n) && held(parts.colx, doubles(192 * (int64_t)blocks)));
 }
 void launch_apply_sym(double *dst, double *X, float *, float4 *rows, const double *, int64_t n, int,
-                      int64_t, int64_t, double, bool, double, unsigned *, cudaStream_t)
+                      int64_t, int64_t, double, bool, double, unsigned *, const SymAlt &alt,
+                      cudaStream_t)
 {
-    note("apply_sym", held(dst, doubles(6 * n)) && held(X, doubles(7 * n)) &&
+    note("apply_sym", (!alt.X3 || held(alt.X3, 80 * (size_t)n)) &&
+                      held(dst, doubles(6 * n)) && held(X, doubles(7 * n)) &&
                           (!rows || held(rows, 64 * (size_t)n)));
 }
 void launch_apply_grp(double *dst, double *X, float *, float4 *rows, const GrpParts &, int64_t n,
-                      const GrpLayout &, int64_t, double, bool, double, unsigned *, cudaStream_t)
+                      const GrpLayout &, int64_t, double, bool, double, unsigned *,
+                      const GrpAlt &alt, cudaStream_t)
 {
-    note("apply_grp", held(dst, doubles(6 * n)) && held(X, doubles(7 * n)) &&
+    note("apply_grp", (!alt.X3 || held(alt.X3, 80 * (size_t)n)) && held(dst, doubles(6 * n)) && held(X, doubles(7 * n)) &&
                           (!rows || held(rows, 64 * (size_t)n)));
 }
 void launch_apply_df64(double *dst, const double *X, const void *, int64_t n, int, int64_t, int64_t,

@@ -95,3 +95,15 @@ def test_the_flags_choose_the_kernel_they_name(fake_library, form, n):
         with Run(fake_library, pair_mode=sk.PAIRS_SYMMETRIC, flags=flag, **FORMS[form]) as r:
             log = r.evolve(n, 2.0 ** -8, 2)
         assert [k for k in log if k.endswith("weak") and not k.startswith("prep")] == [kernel], log
+
+
+@pytest.mark.parametrize("n,order", [(1000, 2), (2999, 4), (4100, 2), (14000, 2)])
+@pytest.mark.parametrize("form", FORMS)
+def test_a_weak_step_launches_the_kernels_for_every_pair_too(fake_library, form, n, order):
+    # the device chooses between the two; one launch of each per sub-step
+    with Run(fake_library, pair_mode=sk.PAIRS_SYMMETRIC, **FORMS[form]) as r:
+        log = r.evolve(n, 2.0 ** -8, order, 2)
+    weak = [k for k in log if k in ("weak", "grp_weak")]
+    every = [k for k in log if k.startswith("every_")]
+    assert len(weak) == len(every) == 2 * (3 if order == 4 else 1)
+    assert len(set(every)) == 1 and ("df64" in every[0]) == (form == "df64")
