@@ -181,6 +181,36 @@ DW_HD double dw_to_double(dw x)
     return (x.h != 0.0f ? h : 0.0) + (x.l != 0.0f ? l : 0.0);
 }
 
+DW_HD float weak_float(uint32_t u)
+{
+#if defined(__CUDA_ARCH__)
+    return __uint_as_float(u);
+#else
+    float f;
+    std::memcpy(&f, &u, 4);
+    return f;
+#endif
+}
+
+// d as the nearest float and the float nearest to the rest, off the FP64 pipe
+// (a conversion instruction costs as much as an FP64 one): |d| in [2^-126,
+// 2^127); below, 0; above, infinity (NaN too).
+DW_HD dw dw_from_double(double d)
+{
+    const uint64_t u = (uint64_t)fpb_bits(d), r = u + (1u << 28);
+    const uint32_t hi = (uint32_t)(u >> 32), he = hi & 0x7ff00000u, sign = hi & 0x80000000u;
+    if (!(he - 0x38100000u < 0x47e00000u - 0x38100000u))
+        return {he < 0x38100000u ? 0.0f : weak_float(0x7f800000u), 0.0f};
+    const uint32_t h = (((uint32_t)(r >> 29) ^ 0x40000000u) & 0x7fffffffu) | sign;
+    // +-2^e of the exponent, and the 29 bits below h's as a signed integer
+    const float e = weak_float((((hi << 3) ^ 0x40000000u) & 0x7f800000u) | sign);
+    const float l = (float)(int32_t)((uint32_t)u << 3);
+    return {weak_float(h), fmul(fmul(l, 0x1p-55f), e)};
+}
+
+// h + l as a double, off the FP64 pipe but for the sum
+DW_HD double dw_double(dw x) { return f2d(x.h) + f2d(x.l); }
+
 // Part of a pair's increments that do not depend on which particle takes
 // them: Q (FP64) multiplies the separation, K the small terms.
 struct WeakPair {

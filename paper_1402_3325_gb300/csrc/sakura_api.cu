@@ -802,6 +802,11 @@ bool sym_path(int64_t n)
 // (2; 4; 8 per warp; the general tile kernel) on 152 SMs: 256 bodies (49; 51;
 // 66; 83), 320 (56; 54; 68; 136), 512 (120; 90; 90; 135), 576 (-; 107; 110;
 // 135), 760 (-; 146; 113; 155), 928 (-; -; 151; 167); 1024 (-; -; 190; 175).
+// It has no prep kernel that could choose: runs of mostly strong pairs take it
+// too, which costs them up to 1.1 times the kernels for every pair up to 512
+// bodies and 1.1 to 1.5 beyond (double-word 1.2 to 1.9: 512 bodies 45 us
+// against 37, 928 91 against 58); the choice would cost every run 3 us and
+// every step 2.
 int weak_small_steps(int64_t n)
 {
     if (g.cfg.grid_blocks > 0 || (g.cfg.flags & SAKURA_FLAG_TILES) || !sym_path(n)) return 0;

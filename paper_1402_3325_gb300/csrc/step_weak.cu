@@ -68,13 +68,17 @@ struct StrongCount {
 };
 
 // Solve of 32 strong pairs (i, j), one per lane, from the drifted state; the
-// twelve products m_j d, -m_i d to out[lane].  FP64: the FP64 solver, seeded
-// from the float copy of the state.  Double-word: the double-word solver for
-// the pairs it admits, the FP64 solver from the analytic guess for the
-// others.  Mixed: the FP32 solver for the pairs its class rule admits, the
-// seeded FP64 solver for the others.  Guess, learned: the FP64 iteration from
-// that guess (the network's weights read from global memory: a batch in a
-// hundred steps or so needs them).
+// increments over m to out[lane][0..5], m_j and -m_i to [6] and [7] (their
+// products are formed by the FMAs that add them to the sums).  FP64: the FP64
+// solver, seeded from the float copy of the state.  Double-word: the
+// double-word solver for the pairs it admits, the FP64 solver from the
+// analytic guess for the others; its operands are converted on the integer
+// pipe (with conversion instructions, as many as 42 FP64-pipe instructions of
+// a pair, and products of their own a step of 800 bodies whose pairs are all
+// strong took 110 us, now 81; FP64 124 -> 112).  Mixed: the FP32 solver for
+// the pairs its class rule admits, the seeded FP64 solver for the others.
+// Guess, learned: the FP64 iteration from that guess (the network's weights
+// read from global memory: a batch in a hundred steps or so needs them).
 template <int MODE>
 __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool valid, int i, int j,
                                                       int weight, double (*out)[12],
@@ -108,10 +112,10 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
         if (valid) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                r[q] = split_dw(rr[q]);
-                v[q] = split_dw(vv[q]);
+                r[q] = dw_from_double(rr[q]);
+                v[q] = dw_from_double(vv[q]);
             }
-            m = split_dw(mi + mj);
+            m = dw_from_double(mi + mj);
             o = dw_phase1(r, v, m, a.ptau32, a.t32, a.guess);
         }
         const bool big = __any_sync(0xffffffffu, o.ok && fabsf(o.x) > 0x1p-8f);
@@ -120,7 +124,7 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
                                               split_dw(a.post * a.tau), o.s, big, dd, evals);
         if (solved) {
 #pragma unroll
-            for (int q = 0; q < 6; ++q) d[q] = (double)dd[q].h + (double)dd[q].l;
+            for (int q = 0; q < 6; ++q) d[q] = dw_double(dd[q]);
         }
         need64 = valid && !solved;
         cnt.iters = o.iters + evals;
@@ -196,10 +200,9 @@ __device__ __noinline__ StrongCount weak_strong_solve(const StepArgs &a, bool va
     }
     if (valid) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            out[lane][q] = mj * d[q];
-            out[lane][6 + q] = -mi * d[q];
-        }
+        for (int q = 0; q < 6; ++q) out[lane][q] = d[q];
+        out[lane][6] = mj;
+        out[lane][7] = -mi;
     }
     return cnt;
 }
@@ -326,8 +329,9 @@ __device__ __forceinline__ void weak_tile(const StepArgs &a, const WeakStep &ws,
                 if (strong) {
 #pragma unroll
                     for (int q = 0; q < 6; ++q) {
-                        s.sacc[q][lane] += s.res[lane][q];
-                        if (!diag) s.sacc[6 + q][c] += s.res[lane][6 + q];
+                        const double x = s.res[lane][q];
+                        s.sacc[q][lane] = fma(s.res[lane][6], x, s.sacc[q][lane]);
+                        if (!diag) s.sacc[6 + q][c] = fma(s.res[lane][7], x, s.sacc[6 + q][c]);
                     }
                 }
                 __syncwarp();
@@ -398,7 +402,7 @@ __global__ void __launch_bounds__(128, 3)
                 const int64_t slot = lane < 6 ? (int64_t)J * Smax + h : (int64_t)I * Smax + h;
                 const int c = lane < 6 ? lane : lane - 6;
                 double *dst = a.partial + (slot * 6 + c) * n + (lane < 6 ? i : j);
-                *dst += res[r0 + e][lane];
+                *dst = fma(res[r0 + e][lane < 6 ? 6 : 7], res[r0 + e][c], *dst);
             }
         }
     };
@@ -574,10 +578,14 @@ __global__ void __launch_bounds__(kFp64GrpWarps * 32, 3)
             for (int e = m0; e < m1; ++e) {
                 const int2 q = s.queue[e - base];
                 const int i = q.x, j = q.y & 0xffffff, cb = q.y >> 24;
-                if (lane < 6)
-                    rs[wib][lane][i & 31] += res[e - r0][lane];
-                else if (lane < 12 && (i >> 5) != (j >> 5))
-                    cs[wib][cb][lane - 6][j & 31] += res[e - r0][lane];
+                const double *r = res[e - r0];
+                if (lane < 6) {
+                    double &x = rs[wib][lane][i & 31];
+                    x = fma(r[6], r[lane], x);
+                } else if (lane < 12 && (i >> 5) != (j >> 5)) {
+                    double &x = cs[wib][cb][lane - 6][j & 31];
+                    x = fma(r[7], r[lane - 6], x);
+                }
             }
             __syncthreads();
         }
@@ -786,7 +794,11 @@ __global__ void __launch_bounds__(128, PER_SM)
         for (int e = 0; e < m; ++e) {
             const int2 q = s.queue[e0 + e];
             const int i = q.x, j = q.y & 0xffffff;
-            if (lane < (diag ? 6 : 12)) sacc[lane][(lane < 6 ? i : j) & 31] += sh.res[r0 + e][lane];
+            if (lane < (diag ? 6 : 12)) {
+                const double *r = sh.res[r0 + e];
+                double &x = sacc[lane][(lane < 6 ? i : j) & 31];
+                x = fma(r[lane < 6 ? 6 : 7], r[lane < 6 ? lane : lane - 6], x);
+            }
         }
     };
     {
