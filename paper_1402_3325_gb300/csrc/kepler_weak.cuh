@@ -147,22 +147,25 @@ DW_HD double square_exact(float y)
     return fpb_double((int64_t)((p << (6u - n)) + ((uint64_t)e << 52)));
 }
 
-// a b for normal a, b and a normal product, rounded to nearest (ties up), on
-// the integer pipe: the upper 74 bits of the 106-bit product of the
-// significands (of the lowest partial product only its upper word, an error
-// below 2^-70), normalised and rounded.
+// a b for normal a, b and a normal product, rounded to nearest even, on the
+// integer pipe: the 106-bit product of the significands, normalised and
+// rounded.
 DW_HD double mul_soft(double a, double b)
 {
     const uint64_t A = (uint64_t)fpb_bits(a), B = (uint64_t)fpb_bits(b);
     const uint32_t ah = (uint32_t)(A >> 32), al = (uint32_t)A;
     const uint32_t bh = (uint32_t)(B >> 32), bl = (uint32_t)B;
     const uint32_t ma = (ah & 0xfffffu) | 0x100000u, mb = (bh & 0xfffffu) | 0x100000u;
-    const uint64_t W = (uint64_t)al * mb + ((uint64_t)ma * bl + (((uint64_t)al * bl) >> 32));
+    const uint64_t L = (uint64_t)al * bl;
+    const uint64_t W = (uint64_t)al * mb + ((uint64_t)ma * bl + (L >> 32));
     const uint64_t H = (uint64_t)ma * mb + (W >> 32);  // in [2^40, 2^42)
     const uint32_t wl = (uint32_t)W, hl = (uint32_t)H, hh = (uint32_t)(H >> 32);
     const uint32_t n = hh >> 9, sh = 12u - n;
     const uint32_t rh = (hh << sh) | (hl >> (32u - sh)), rl = (hl << sh) | (wl >> (32u - sh));
-    const uint32_t up = (wl << sh) >> 31;
+    // the bits below the significand: the upper one, and whether the rest is
+    // more than nothing or the significand odd
+    const uint32_t t = wl << sh;
+    const uint32_t up = (t >> 31) & (uint32_t)(((t << 1) | (uint32_t)L | (rl & 1u)) != 0u);
     // the significand's hidden bit adds one to the exponent
     const uint32_t e = (ah & 0x7ff00000u) + (bh & 0x7ff00000u) + (n << 20) - (1024u << 20);
     const uint64_t r = (((uint64_t)(rh + e) << 32) | rl) + up;
@@ -426,7 +429,7 @@ DW_HD void weak_add(const WeakParticle &a, const WeakParticle &b, const WeakDiff
     const dw xd[3] = {dw_split0(d.x[0]), dw_split0(d.x[1]), dw_split0(d.x[2])};
     WeakPair o;
     weak_solve(d.r2, d.r2d, xd, d.w, dwu_add(a.mh, b.mh), o);
-    // on the integer pipe (about 20 instructions): 3 % of a step on tiles at
+    // on the integer pipe (about 25 instructions): 3 % of a step on tiles at
     // 4000 bodies, 1 % in row groups at 16384.  The other two multiplies (y^3,
     // z^2) there too gained nothing more.
     const double qj = mul_soft(b.mt, o.Q), qi = mul_soft(a.mt, o.Q);
