@@ -103,10 +103,10 @@ EMU_ITER_MULS = 10
 
 # a weakly perturbed pair (csrc/kepler_weak.cuh), which nearly every pair of
 # these workloads is: FP64 separation 3, r0^2 5, 1 - r0^2 y^2 2, the leading
-# factor 3, its products with the two masses 2 (on the integer pipes) and the
+# factor 4, its products with the two masses 2 (on the integer pipes) and the
 # two velocity sums 12.  Its corrections, in double-word FP32 arithmetic, and
 # the FP64 solves of the other pairs are not counted.
-C_WEAK = 27
+C_WEAK = 28
 EMU_WEAK_MULS = 2
 
 
@@ -708,6 +708,12 @@ def _roofline(workload, form, pairs, guess, n, small, m):
     solves = n * (n - 1) * m["solves_per_pair"]
     pair_ms = m["pair_kernel_ms"]
     achieved = solves * flops / (pair_ms * 1e-3) / 1e12 if flops and pair_ms > 0 else None
+    counts = {"kepler_evals_per_solve": kbar, "carried_share": carried,
+              "iteration_lane_efficiency": m["iteration_lane_efficiency"]}
+    if weak and form == "fp64" and guess != "fp32":
+        # statistics make the library iterate every pair from these guesses:
+        # not the kernel that is timed
+        counts = dict.fromkeys(counts)
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if achieved else None,
             "traffic": _profiled_traffic(workload, kname),
@@ -717,13 +723,33 @@ def _roofline(workload, form, pairs, guess, n, small, m):
                 (1.0 - share if form == "mixed" else 1.0) *
                 _integer_pipe_flops(kname, guess, kbar, mixed=form == "mixed")
                 if form in ("fp64", "mixed") and pipe.startswith("fp64") and not small else 0.0),
-            "kepler_evals_per_solve": kbar,
-            "carried_share": carried, "iteration_lane_efficiency": m["iteration_lane_efficiency"],
-            "solves_per_step": solves, "pair_kernel_ms": pair_ms,
+            **counts, "solves_per_step": solves, "pair_kernel_ms": pair_ms,
             "pair_kernel_share": pair_ms / m["ms_per_step"],
             "pair_kernel_timing": ("CUDA events around each pair-kernel launch on the library"
                                    " stream, in a second pass of the same K steps with L2"
                                    " flushed before each call")}
+
+
+def _launches(sk, n, form, pairs, mixed_rule, guess, steps, per_call, small):
+    """Kernels that the library launches for `steps` steps in calls of
+    per_call steps: one per call for small systems; two per step where each
+    block prepares its own particles; otherwise a pair and an apply kernel per
+    step, a second pair kernel where weakly perturbed pairs have their own (the
+    one not chosen returns at once), and a prep kernel per step, or per call
+    where every apply kernel drifts for the next step."""
+    if small:
+        return steps // per_call
+    literal = mixed_rule != "hyp"
+    on_tiles = bool(EXTRA_FLAGS & sk.FLAG_TILES) or (
+        not EXTRA_FLAGS & sk.FLAG_GROUPS and n <= (4095 if literal else 640))
+    weak = pairs == "symmetric" and (form in ("fp64", "df64") or
+                                     (literal and guess == "fp32"))
+    if weak and n <= 928 and not EXTRA_FLAGS:
+        return 2 * steps
+    step = 3 if weak else 2
+    if pairs == "symmetric" and (form != "mixed" or on_tiles):
+        return (steps // per_call) * (1 + step * per_call)
+    return (1 + step) * steps
 
 
 def _measure(args, sk, s, device, stream, flush, guess, opts, per_call, clocks=None,
@@ -967,7 +993,6 @@ def main():
             dist.destroy_process_group()
         return 0
 
-    symmetric = args.pairs == "symmetric" and args.form in ("fp64", "df64")
     roof = _roofline(args.workload, args.form, args.pairs, args.guess, n, small, m)
     solves = n * (n - 1) * m["solves_per_pair"]
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
@@ -995,12 +1020,8 @@ def main():
                                    " call in one launch" if small else
                                    "drift, pair and apply kernels per step"),
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
-            # small systems: one launch per call; symmetric FP64 tiles: a
-            # prep kernel per call, then a pair and an apply kernel per step
-            # (each apply drifts for the next); otherwise prep, pair, apply
-            "gpu_launches": ((args.steps // per_call) if small else
-                             (args.steps // per_call) * (1 + 2 * per_call)
-                             if (args.form == "fp64" and symmetric) else 3 * args.steps),
+            "gpu_launches": _launches(sk, n, args.form, args.pairs, args.mixed_rule, args.guess,
+                                      args.steps, per_call, small),
             "solves_per_pair": m["solves_per_pair"],
             "roofline": roof, "clocks": clocks.summary()}
     if e2e is not None:
