@@ -74,7 +74,9 @@ extern "C" {
 /* Initial value of the Kepler iteration.  In the symmetric second-order FP64
  * step, pairs that move by less than 2^-5 of their separation need none: they
  * are solved as one FP64 term and double-word corrections, to the same
- * accuracy.  With SAKURA_GUESS_FP32 they count as one evaluation, carried;
+ * accuracy.  (Above 928 bodies a call whose pairs mostly move by more, as a
+ * sample of the state before it tells, solves every pair by the iteration.)
+ * With SAKURA_GUESS_FP32 they count as one evaluation, carried;
  * with the other guesses every pair iterates when SAKURA_FLAG_STATS is set
  * (or kepler_max_iter < 8 or kepler_tol < 1), so that the counts are the
  * guess's.                                                                  */

@@ -633,9 +633,9 @@ int step_device_fp64_grp(const double *src, double *dst, const double *masses, i
 
 // Unordered pairs once (Newton's third law): systolic 32 x 32 tiles; df64:
 // the pair solves in double-word arithmetic (step_df64.cu).
-// prepped: X (and X32) already hold this sub-step's drifted state, written
-// by the previous apply kernel (FP64 form only); fuse: the apply kernel also
-// applies the next sub-step's drift next_drift and writes its X (and X32).
+// prepped: X (and X32 or X3, and the weak rows) already hold this sub-step's
+// drifted state, written by the previous apply kernel; fuse: the apply kernel
+// also applies the next sub-step's drift next_drift and writes them (fusable).
 int step_device_sym(const double *src, double *dst, const double *masses, int64_t n, double dt,
                     int order, bool df64, bool mixed, bool weak, bool prepped, bool fuse,
                     double next_drift)

@@ -378,7 +378,6 @@ __global__ void __launch_bounds__(kGrpWarps * 32, 2)
     const int64_t B = gridDim.x;
     const int64_t b = blockIdx.x;
     const float *X32 = ma.X32;
-    const KeplerParams kp{a.tol, a.max_iter, a.bisection};
     unsigned status = 0;
     long long it_sum = 0, slots = 0, fallbacks = 0, n32 = 0, carries = 0;
     int it_max = 0;

@@ -19,16 +19,16 @@
 // bodies 1105 -> 766, double-word 949 -> 351.
 //
 // Bound: the FP64 pipe (16 FP64 instructions per pair and 16 cycles each)
-// and the issue slots (950 instructions per pair and warp) nearly alike: ncu
-// at 8192 bodies (black hole), 67 % and 63 %, neither full with the 12 warps
+// and the issue slots (966 instructions per pair and warp) nearly alike: ncu
+// at 8192 bodies (black hole), 70 % and 62 %, neither full with the 12 warps
 // per SM that 168 registers leave.  ms per step: 16384 bodies (black hole)
-// 20.36 -> 5.08 in row groups; Plummer 1024 0.109 -> 0.043, 2048 0.358 ->
-// 0.103, 4000 1.30 -> 0.332 (the kernels of step_sym.cu and step_grp.cu with
+// 20.36 -> 5.16 in row groups; Plummer 1024 0.109 -> 0.043, 2048 0.358 ->
+// 0.103, 4000 1.30 -> 0.313 (the kernels of step_sym.cu and step_grp.cu with
 // the seed before); the double-word form, 16384 bodies with binaries: 8.29 ->
-// 5.45 (step_df64.cu before: every pair in 1922 double-word flops); the mixed
-// form's literal rule, 5003 bodies: 2.11 -> 0.55; the default guess, 2999
-// bodies, a fourth-order step on host arrays: 3.26 -> 0.74; the learned
-// guess, 8192 bodies with binaries: 7.06 -> 1.55.
+// 5.46 (step_df64.cu before: every pair in 1922 double-word flops); the mixed
+// form's literal rule, 5003 bodies: 2.11 -> 0.57; the default guess, 2999
+// bodies, a fourth-order step on host arrays: 3.26 -> 0.75; the learned
+// guess, 8192 bodies with binaries: 7.06 -> 1.62.
 #include <cuda_runtime.h>
 
 #include "kepler_df64.cuh"
@@ -719,7 +719,8 @@ __global__ void prep_weak_kernel(const double *state, const double *mass, double
 // sums of the rows' particles, slot (I, h) with the column sums of the
 // columns'.  Within the block layout indices are local: rows 0 .. 31, columns
 // 32 .. 63 (a diagonal tile: 0 .. 31).  PER_SM 2: up to 255 registers, no
-// spills; 3 where the grid needs three blocks per SM to be resident at once.
+// spills but 44 bytes of the learned guess's; 3 where the grid needs three
+// blocks per SM to be resident at once.
 // Four steps of a run and a copy of the state before them in us, pair kernel
 // on general tiles with drift, pair and apply kernels before -> now: 128
 // bodies 70 -> 43, 512 135 -> 90, 760 155 -> 114, 928 181 -> 151; where most
